@@ -31,6 +31,7 @@
 #include "igamg_internal.h"
 #include "kernels.cuh"
 #include "kernels_adv.cuh"
+#include "kernels_patch.cuh"
 #include "krylov.h"
 
 using namespace igamg;
@@ -199,6 +200,7 @@ struct TypedLevel {
   T* cinv = nullptr;
   T* cinv8 = nullptr;
   Xfer<T> tp{}, tq{};            // transfer from level l-1 into level l (l >= 1)
+  PatchTab<T> X{};               // staged patch solves: records and inverses in their layout
   T *U = nullptr, *F = nullptr, *R = nullptr;
   unsigned* prog = nullptr;      // pipelined sweep: colour steps finished per tile
 };
@@ -231,6 +233,9 @@ struct LevelCommon {
   // ntx = 0 where the level uses one launch per colour
   int tw = 0, ntx = 0, nty = 0;
   int *tile_list = nullptr, *tile_off = nullptr, *tile_n8 = nullptr;
+  bool staged = false;          // staged patch solves (kernels_patch.cuh), one launch per colour
+  int *gcls = nullptr, *wrow = nullptr;   // PatchGrids, device copies
+  std::vector<ColourGrid> grids;  // per colour (empty: the level does not suit the staged kernels)
   int lpr = 1;                  // lanes per local row of an 8-DOF patch in the colour kernels
   int tpb = 0;                  // threads per block of the colour kernels (0: colour_block())
   int ch = 4;                   // multiply-add chains per row in the one-lane FP64 colour kernel (4 or 2;
@@ -411,10 +416,40 @@ int do_residual(igamg_handle* h, int l, const T* U, const T* F, T* R, double* no
   return launch_check();
 }
 
+// One sweep of staged patch solves, one launch per colour.  Each launch may begin while the one
+// before it runs (programmatic dependent launch): it fetches its records and inverses, which no
+// kernel writes, then waits for the earlier launches to finish (dependency_wait).
+constexpr int kPatchThreads = 64;
+template <int P, typename T>
+int do_smooth_staged(igamg_handle* h, int l, T* U, const T* F, cudaStream_t s) {
+  auto& lc = h->lc[l];
+  auto& tl = typed<T>(h).lev[l];
+  const int gpb = kPatchThreads / PatchShape<P>::LW, smg = group_entries<P>(lc.maxl);
+  cudaLaunchConfig_t cfg = {};
+  cfg.blockDim = dim3(kPatchThreads);
+  cfg.dynamicSmemBytes = (size_t)gpb * smg * sizeof(limb_t<T>);
+  cfg.stream = s;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  for (const ColourGrid& C : lc.grids) {
+    const int ng = colour_groups<P>(C);
+    if (ng == 0) continue;
+    cfg.gridDim = dim3((unsigned)((ng + gpb - 1) / gpb));
+    const cudaError_t e = tl.X.ext ? cudaLaunchKernelEx(&cfg, k_patch_colour<P, T, true>, tl.L, tl.X, U, F, C, ng, smg)
+                                   : cudaLaunchKernelEx(&cfg, k_patch_colour<P, T, false>, tl.L, tl.X, U, F, C, ng, smg);
+    if (e != cudaSuccess) { g_err = cudaGetErrorString(e); return IGAMG_ECUDA; }
+  }
+  return IGAMG_OK;
+}
+
 template <typename T>
 int do_smooth(igamg_handle* h, int l, T* U, const T* F, cudaStream_t s) {
   auto& lc = h->lc[l];
   auto& tl = typed<T>(h).lev[l];
+  if (lc.staged) return h->prob.p == 2 ? do_smooth_staged<2, T>(h, l, U, F, s) : do_smooth_staged<3, T>(h, l, U, F, s);
   size_t shm = (size_t)(kBlock / 32) * lc.maxl * sizeof(T);
   if (h->prob.smoother == IGAMG_MULT && split_colour(tl.L.srow != nullptr)) {
     size_t shm16 = (size_t)16 * lc.maxl * sizeof(T);
@@ -845,6 +880,9 @@ void mix_descriptors(int n, igamg_handle** hs, double** Us, const double** Fs, c
         d.nloc = lc.nloc;
         d.maxl = lc.maxl;
         d.lpr = 1;            // one lane per row: the batch launches are throughput-bound
+        d.staged = lc.staged ? 1 : 0;
+        d.X = tl.X;
+        for (size_t c = 0; c < lc.grids.size() && c < kMaxColours; ++c) d.grid[c] = lc.grids[c];
         for (int c = 0; c < lc.n_colours && c < kMaxColours; ++c) {
           d.first[c] = lc.colour_off[c];
           d.cnt[c] = lc.colour_off[c + 1] - lc.colour_off[c];
@@ -884,16 +922,28 @@ int batch_launches(igamg_handle** all, const std::vector<int>& idx, const std::v
   };
   auto smooth = [&](int t) {
     const int C = hs[0]->lc.back().n_colours;
-    const size_t shm = (size_t)wpb * max_over(t, 1, [&](int i, int l) { return hs[i]->lc[l].maxl; }) * sizeof(double);
+    // shared memory per group of a staged level, and per block of any level
+    auto entries = [&](int i, int l) {
+      const int m = hs[i]->lc[l].maxl;
+      return !hs[i]->lc[l].staged ? 0 : (p == 2 ? group_entries<2>(m) : group_entries<3>(m));
+    };
+    const int smg = (int)max_over(t, 1, entries), gpb = p == 2 ? tpb / PatchShape<2>::LW : tpb / PatchShape<3>::LW;
+    const size_t shm = sizeof(double) * std::max((size_t)gpb * smg, (size_t)wpb * max_over(t, 1, [&](int i, int l) {
+      return hs[i]->lc[l].staged ? 0 : hs[i]->lc[l].maxl;
+    }));
+    const bool ext = hs[0]->d.lev.back().X.ext != nullptr;
     for (int c = 0; c < C; ++c) {
       unsigned nb = max_over(t, 1, [&](int i, int l) {
         const auto& lc = hs[i]->lc[l];
+        if (lc.staged) return ((p == 2 ? colour_groups<2>(lc.grids[c]) : colour_groups<3>(lc.grids[c])) + gpb - 1) / gpb;
         const int ppw = 4;
         const int n8 = lc.n8[c], ngen = lc.colour_off[c + 1] - lc.colour_off[c] - n8;
         return (n8 + ppw * wpb - 1) / (ppw * wpb) + (ngen + wpb - 1) / wpb;
       });
-      if (p == 2) k_mix_colour<2, double><<<dim3(nb, ns), tpb, shm, s>>>(A[t], c);
-      else k_mix_colour<3, double><<<dim3(nb, ns), tpb, shm, s>>>(A[t], c);
+      if (p == 2 && !ext) k_mix_colour<2, double, false><<<dim3(nb, ns), tpb, shm, s>>>(A[t], c, smg);
+      else if (p == 2) k_mix_colour<2, double, true><<<dim3(nb, ns), tpb, shm, s>>>(A[t], c, smg);
+      else if (!ext) k_mix_colour<3, double, false><<<dim3(nb, ns), tpb, shm, s>>>(A[t], c, smg);
+      else k_mix_colour<3, double, true><<<dim3(nb, ns), tpb, shm, s>>>(A[t], c, smg);
     }
   };
   if (cycle) {
@@ -1620,6 +1670,56 @@ std::vector<double> round_bf16(const std::vector<double>& v) {
   return out;
 }
 
+// The staged patch kernels' records and inverses of level l, made on the device from the uploaded
+// tables (FP64: integer limbs; FP32: the same values, u_y rows with y outer).
+template <int P, typename T>
+int build_patch_tab(igamg_handle* h, int l, TypedLevel<T>& tl) {
+  using S = PatchShape<P>;
+  using E = limb_t<T>;
+  auto& lc = h->lc[l];
+  const auto& lh = h->host.lev[l];
+  const LevelTab<T>& L = tl.L;
+  PatchGrids G;                    // (offsets of the inverses differ between FP64 limbs and FP32)
+  if (!patch_grids(P, lh.sz, lh.pt, L.srow != nullptr, (int)sizeof(E), G)) return IGAMG_EINVAL;
+  PatchTab<T>& X = tl.X;
+  int *wdesc, *wspec, rc;
+  if ((rc = upload_as(h, &wdesc, G.wdesc)) || (rc = upload_as(h, &wspec, G.wspec))) return rc;
+  X.gcls = lc.gcls;
+  X.wrow = reinterpret_cast<const int4*>(lc.wrow);
+  X.wdesc = reinterpret_cast<const int4*>(wdesc);
+  X.by_row = L.srow != nullptr;
+  E *rec, *inv8, *winv;
+  if (L.srow) {
+    const int n = L.n_total - 1;
+    if ((rc = dmalloc(h, (void**)&rec, (size_t)n * S::NREC * sizeof(E)))) return rc;
+    k_patch_records<P, T><<<nblk(n), kBlock, 0, h->stream>>>(n, -1, L.n_ux, L.n_uy, L.srow, rec);
+  } else {
+    const T* src[3] = {L.sx, L.sy, L.sp};
+    const int n = (int)(lh.st.sx.size() / S::RU);
+    if ((rc = dmalloc(h, (void**)&rec, (size_t)3 * n * S::NREC * sizeof(E)))) return rc;
+    for (int k = 0; k < 3; ++k)
+      k_patch_records<P, T><<<nblk(n), kBlock, 0, h->stream>>>(n, k, 0, 0, src[k], rec + (size_t)k * n * S::NREC);
+  }
+  X.rec = rec;
+  if (L.sext) {
+    const int n = L.n_ux + L.n_uy;
+    E* ext;
+    if ((rc = dmalloc(h, (void**)&ext, (size_t)n * S::NEXT * sizeof(E)))) return rc;
+    k_patch_ext<P, T><<<nblk(n), kBlock, 0, h->stream>>>(n, L.n_ux, L.sext, ext);
+    X.ext = ext;
+  }
+  const int n8 = std::max(lh.pt.n_cls8, 1), nw = (int)G.wspec.size() / 4;
+  if ((rc = dmalloc(h, (void**)&inv8, (size_t)n8 * 8 * inv8_ld<T>() * sizeof(E))) ||
+      (rc = dmalloc(h, (void**)&winv, (size_t)std::max(G.winv16, 1) * 16)))
+    return rc;
+  k_patch_inv8<T><<<nblk(n8 * 8), kBlock, 0, h->stream>>>(n8, tl.cinv8, inv8);
+  if (nw > 0)
+    k_patch_winv<T><<<nw, S::LW, 0, h->stream>>>(lc.maxl, reinterpret_cast<const int4*>(wspec), tl.cinv, tl.cinv8, winv);
+  X.inv8 = inv8;
+  X.winv = winv;
+  return launch_check();
+}
+
 // Upload the typed (double or float) copy of every level's tables and workspaces.
 template <typename T>
 int upload_typed(igamg_handle* h, Typed<T>& ty, size_t max_delta) {
@@ -1653,6 +1753,9 @@ int upload_typed(igamg_handle* h, Typed<T>& ty, size_t max_delta) {
         X.nf = Tr.nf; X.nc = Tr.nc; X.c0 = c0; X.f0 = f0; X.pv = pv; X.rv = rv;
       }
     }
+    if (!h->lc[l].grids.empty() &&
+        (rc = p == 2 ? build_patch_tab<2, T>(h, l, tl) : build_patch_tab<3, T>(h, l, tl)))
+      return rc;
     size_t nb = (size_t)lh.sz.n_total * sizeof(T);
     if ((rc = dmalloc(h, (void**)&tl.R, nb))) return rc;
     if ((rc = dmalloc(h, (void**)&tl.U, nb))) return rc;
@@ -1738,13 +1841,18 @@ int tile_capacity(int p, int maxl) {
 //   colour launches, two lanes per patch row  (lpr 2: two patches per warp; 128 or 64)
 //   one block for the whole level             (k_sweep_tiles with one tile of 512 threads)
 //   pipelined tiles of (p + 1) m positions    (k_sweep_tiles, 128 threads, m = 1, 2, 4)
+// Levels that suit the staged patch kernels (kernels_patch.cuh; every level but those whose patches
+// have more than 32 (p = 2) or 64 (p = 3) rows, i.e. p = 3 on 4 x 4 elements) always use those:
+// they were faster than every other form on every level measured (8^2 to 512^2, p = 2 and 3, FP64
+// and FP32, all operator forms: 1.1x on the largest records to 4.7x; figures in that file).  The
+// other forms remain for the levels left over and for the pins below.
 // Each candidate is timed the way solves run it: nu1 sweeps of the level captured into a CUDA
 // graph, replayed after a warm-up (best of three), on the level's zeroed FP64 workspaces (the
 // arithmetic does not depend on the values).  Choices are cached per process by (p, n, per-row
 // records, mapped).  IGAMG_PIPELINE=0 leaves out the tile forms; IGAMG_SWEEP_FORM pins one
 // ("lanes1", "lanes2", "lanes1_b64", "lanes2_b64", "lanes1_b256", "solo", "tiles1", "tiles2",
 // "tiles4").
-struct SweepForm { int lpr = 1, tiles = 0, tpb = 0, ch = 4; };   // tiles: 0 colour launches, -1 one block, m > 0
+struct SweepForm { int lpr = 1, tiles = 0, tpb = 0, ch = 4; bool staged = false; };   // tiles: 0 colour launches, -1 one block, m > 0
 std::map<std::tuple<int, int, int, int>, SweepForm>& form_cache() {
   static std::map<std::tuple<int, int, int, int>, SweepForm> m;
   return m;
@@ -1757,6 +1865,7 @@ std::mutex& form_mutex() {
 }
 
 std::string form_name(const SweepForm& f) {
+  if (f.staged) return "staged";
   if (f.tiles == 0)
     return std::string(f.lpr == 2 ? "lanes2" : "lanes1") + (f.tpb ? "_b" + std::to_string(f.tpb) : "") +
            (f.ch == 2 ? "_c2" : "");
@@ -1770,8 +1879,9 @@ int apply_form(igamg_handle* h, int l, const SweepForm& f) {
   auto& lc = h->lc[l];
   const int p = h->prob.p;
   const PatchTables& pt = h->host.lev[l].pt;
+  lc.staged = f.staged;
   lc.lpr = f.lpr;
-  lc.tpb = f.tpb;
+  lc.tpb = f.staged ? kPatchThreads : f.tpb;
   lc.ch = f.lpr == 1 && f.tiles == 0 ? f.ch : 4;
   lc.ntx = lc.nty = 0;
   if (f.tiles == 0) return IGAMG_OK;
@@ -1877,6 +1987,10 @@ int setup_sweep_forms(igamg_handle* h) {
       else if (w == "solo") f.tiles = -1;
       else if (w.rfind("tiles", 0) == 0) f.tiles = std::max(1, std::atoi(w.c_str() + 5));
       add(f);
+    } else if (!lc.grids.empty() && !env_lanes && !env_mult && !split_colour(h->d.lev[l].L.srow != nullptr)) {
+      SweepForm f;                                             // every level whose patches fit its layout
+      f.staged = true;
+      cands.push_back(f);
     } else if (env_lanes || env_mult) {                        // experiments: one form
       SweepForm f;
       if (env_mult && tiles_ok) f.tiles = std::max(1, std::atoi(env_mult));
@@ -2123,6 +2237,12 @@ int igamg_create(const igamg_problem* prob, void* cuda_stream, igamg_handle** ou
       const auto& pt = lh.pt;
       lc.n_patches = pt.n_patches; lc.maxl = pt.maxl; lc.n_colours = pt.n_colours;
       lc.colour_off = pt.colour_off; lc.n8 = pt.n8;
+      PatchGrids G;
+      if (pr.smoother == IGAMG_MULT && patch_grids(p, lh.sz, pt, !lh.rows.empty(), 8, G)) {
+        for (const PatchGrid& g : G.colour)
+          lc.grids.push_back(ColourGrid{g.a0, g.b0, g.na, g.n8, g.gfirst, g.wfirst, g.nwall});
+        if ((rc = upload_as(h, &lc.gcls, G.gcls)) || (rc = upload_as(h, &lc.wrow, G.wrow))) return fail(rc);
+      }
       if ((rc = upload_as(h, &lc.dofs, pt.dofs)) || (rc = upload_as(h, &lc.cls, pt.cls)) ||
           (rc = upload_as(h, &lc.nloc, pt.nloc)) || (rc = upload_as(h, &lc.d2p_off, pt.d2p_off)) ||
           (rc = upload_as(h, &lc.d2p_idx, pt.d2p_idx)))

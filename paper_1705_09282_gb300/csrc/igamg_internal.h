@@ -86,6 +86,31 @@ struct TileTables {
 };
 void build_tile_tables(const PatchTables& pt, int nint, int tw, TileTables& tt);
 
+// One colour's patches as the staged patch kernels (kernels_patch.cuh) take them (2D): the
+// interior patches, whose neighbourhood lies inside the index range, at positions a0 + i (p+1),
+// b0 + j (p+1), na of them per row of positions, n8 in all, their classes at gcls[gfirst ..] row
+// by row; and the other patches, nwall entries of wdesc / wrow from wfirst.
+struct PatchGrid { int a0 = 1, b0 = 1, na = 0, n8 = 0, gfirst = 0, wfirst = 0, nwall = 0; };
+struct PatchGrids {
+  std::vector<PatchGrid> colour;
+  std::vector<int> gcls;       // interior patches: index into cinv8
+  // other patches, 4 ints each: a | b << 16, offset of its inverse (16-byte units), rows |
+  // velocity rows << 8, 0; and per row (lw rows per patch, 32 at p = 2 and 64 at p = 3) 4 ints:
+  // the row, the offsets of its boxes A | B << 16 in the staged arrays, that of the third box, the
+  // index of its record
+  std::vector<int> wdesc, wrow;
+  // the inverses of those patches, one per class, 4 ints each: class in cinv (or -1 - class in
+  // cinv8), offset (16-byte units), rows | velocity rows << 8, 0; total size in 16-byte units
+  std::vector<int> wspec;
+  int winv16 = 0;
+};
+// Fills G if the level suits those kernels; otherwise returns false.  by_row: records per row, not
+// per class; entry_bytes: 8 (FP64 limbs) or 4.  Checked for every patch, not assumed: the interior
+// patches have the DOFs of their position, no patch has more than lw rows, and every stencil
+// position of every other patch's rows that lies in the domain is inside the patch's staged
+// arrays, every other one inside the margin.
+bool patch_grids(int p, const igamg_sizes& s, const PatchTables& pt, bool by_row, int entry_bytes, PatchGrids& G);
+
 // Row stencils of K_l by row class.  A row's class is the pair of 1D position classes
 // of its two indices (cls1 below): positions within T of either end are their own class,
 // all others share the translation-invariant interior class.  Coefficients of neighbours

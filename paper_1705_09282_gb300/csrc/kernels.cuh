@@ -980,154 +980,5 @@ __global__ void k_curl_update(LT L, const double* __restrict__ dcoef, const doub
   }
 }
 
-// ---- lockstep batches of any mesh sizes: one launch per V-cycle step over every solve -------
-// The solves of a batch share p and the cycle shape but may differ in mesh size and number
-// of grids.  Their V-cycles are aligned from the finest grid down: at depth t (0 = finest) a
-// solve with L grids is on its level L - 1 - t.  A launch covers up to kMixChunk solves of any
-// sizes (blockIdx.y = solve), their descriptors for that depth in the kernel parameters;
-// larger batches are cut into chunks that run as parallel branches of one graph.  A block
-// whose solve is converged, past its coarsest level, not on a level that takes part in the
-// step, or beyond that solve's work, returns at once.
-template <typename T>
-struct MixLevel {
-  int level;                      // level index in the solve's hierarchy, -1 past its coarsest
-  int lpr;                        // lanes per 8-DOF patch row of the level's colour kernel
-  LevelTab<T> L, Lc;              // this level and (level >= 1) the next coarser one
-  Xfer<T> tp, tq;                 // transfers between Lc and L
-  const T *cinv, *cinv8, *kinv;   // local inverses; kinv: the coarsest level's dense inverse
-  T *U, *F, *R, *Uc, *Fc;
-  const int *dofs, *cls, *nloc;
-  int maxl;
-  int first[kMaxColours], n8[kMaxColours], cnt[kMaxColours];
-  double* part;                   // residual partials (two per block of 256 rows)
-  double* norm2;                  // ||F - K U||^2 of the finest level
-  const int* active;              // 1 while the solve is iterating
-};
-
-constexpr int kMixChunk = 24;     // solves per launch (descriptors in the kernel parameters)
-
-template <typename T>
-struct MixArgs {
-  int count;
-  MixLevel<T> s[kMixChunk];
-};
-
-template <int P, typename T>
-__global__ void __launch_bounds__(256) k_mix_colour(const __grid_constant__ MixArgs<T> A, int c) {
-  const MixLevel<T>& d = A.s[blockIdx.y];
-  if (d.level < 1 || !*d.active) return;
-  const int wpb = blockDim.x >> 5, ppw = d.lpr == 2 ? 2 : 4;
-  const int n8 = d.n8[c], ngen = d.cnt[c] - n8;
-  const int nb8 = (n8 + ppw * wpb - 1) / (ppw * wpb), nbg = (ngen + wpb - 1) / wpb;
-  if ((int)blockIdx.x >= nb8 + nbg) return;
-  const LevelTab<T> L = d.L;
-  T* U = d.U;
-  const T* F = d.F;
-  const int *dofs = d.dofs, *cls = d.cls, *nloc = d.nloc;
-  const T *cinv = d.cinv, *cinv8 = d.cinv8;
-  const int maxl = d.maxl, first = d.first[c];
-  // the block walks the solve's blocks with the grid's stride (a descriptor read serves
-  // several rounds of patches)
-  for (int b = blockIdx.x; b < nb8 + nbg; b += gridDim.x) {
-    if (d.lpr == 2)
-      mult_colour_block<P, T, 2>(L, U, F, dofs, cls, cinv, cinv8, nloc, maxl, first, n8, ngen, nb8, b);
-    else
-      mult_colour_block<P, T, 1, 2>(L, U, F, dofs, cls, cinv, cinv8, nloc, maxl, first, n8, ngen, nb8, b);
-  }
-}
-
-// R = F - K U with per-block partials; any_level: also for solves on their coarsest level
-// (the finest level of a one-grid solve, for its norm)
-template <int P, typename T>
-__global__ void __launch_bounds__(256) k_mix_residual(const __grid_constant__ MixArgs<T> A,
-                                                      int any_level) {
-  __shared__ double sh[32];
-  const MixLevel<T>& d = A.s[blockIdx.y];
-  if (d.level < (any_level ? 0 : 1) || !*d.active) return;
-  const LevelTab<T> L = d.L;
-  if ((int)(blockIdx.x * blockDim.x) >= L.n_total - 1) return;
-  int g = blockIdx.x * blockDim.x + threadIdx.x;
-  double r2 = 0.0, mp = 0.0;
-  if (g < L.n_total - 1) {
-    T r = d.F[g] - row_KU<P, T, 2, 2>(L, d.U, g);
-    d.R[g] = r;
-    r2 = (double)r * (double)r;
-    int off = g - L.n_ux - L.n_uy;
-    if (off >= 0) mp = (double)mean_coef<P>(L, off) * (double)d.U[g];
-  }
-  double s1 = block_sum(r2, sh);
-  double s2 = block_sum(mp, sh);
-  if (threadIdx.x == 0) { d.part[2 * blockIdx.x] = s1; d.part[2 * blockIdx.x + 1] = s2; }
-}
-
-template <typename T>
-__global__ void k_mix_residual_finish(const __grid_constant__ MixArgs<T> A, int any_level,
-                                      int want_norm, int rows_per_part) {
-  __shared__ double sh[32];
-  const MixLevel<T>& d = A.s[blockIdx.x];
-  if (d.level < (any_level ? 0 : 1) || !*d.active) return;
-  const int n_total = d.L.n_total, nparts = (n_total - 1 + rows_per_part - 1) / rows_per_part;
-  double a = 0.0, c = 0.0;
-  for (int i = threadIdx.x; i < nparts; i += blockDim.x) { a += d.part[2 * i]; c += d.part[2 * i + 1]; }
-  double s1 = block_sum(a, sh);
-  double s2 = block_sum(c, sh);
-  if (threadIdx.x == 0) {
-    double rl = (double)d.F[n_total - 1] - s2;
-    d.R[n_total - 1] = (T)rl;
-    if (want_norm) *d.norm2 = s1 + rl * rl;
-  }
-}
-
-// coarse F = P^T R
-template <typename T>
-__global__ void k_mix_restrict(const __grid_constant__ MixArgs<T> A) {
-  const MixLevel<T>& d = A.s[blockIdx.y];
-  if (d.level < 1 || !*d.active) return;
-  int g = blockIdx.x * blockDim.x + threadIdx.x;
-  const int nc = d.Lc.n_total;
-  if (g >= nc) return;
-  d.Fc[g] = (g == nc - 1) ? d.R[d.L.n_total - 1] : restrict_elem(d.L, d.Lc, d.tp, d.tq, d.R, g);
-}
-
-// U += P Uc
-template <typename T>
-__global__ void k_mix_prolong_add(const __grid_constant__ MixArgs<T> A) {
-  const MixLevel<T>& d = A.s[blockIdx.y];
-  if (d.level < 1 || !*d.active) return;
-  int g = blockIdx.x * blockDim.x + threadIdx.x;
-  const int nf = d.L.n_total;
-  if (g >= nf) return;
-  d.U[g] += (g == nf - 1) ? d.Uc[d.Lc.n_total - 1] : prolong_elem(d.L, d.Lc, d.tp, d.tq, d.Uc, g);
-}
-
-template <typename T>
-__global__ void k_mix_zero(const __grid_constant__ MixArgs<T> A) {
-  const MixLevel<T>& d = A.s[blockIdx.y];
-  if (d.level < 1 || !*d.active) return;
-  int g = blockIdx.x * blockDim.x + threadIdx.x;
-  if (g < d.L.n_total) d.U[g] = T(0);
-}
-
-// U = K_0^{-1} F for the solves on their coarsest level at this depth, one block per solve
-template <typename T>
-__global__ void k_mix_coarse(const __grid_constant__ MixArgs<T> A) {
-  const MixLevel<T>& d = A.s[blockIdx.x];
-  if (d.level != 0 || !*d.active) return;
-  extern __shared__ unsigned char smem_raw[];
-  T* g = reinterpret_cast<T*>(smem_raw);
-  const int n = d.L.n_total;
-  for (int i = threadIdx.x; i < n; i += blockDim.x) g[i] = d.F[i];
-  __syncthreads();
-  int lane = threadIdx.x & 31, nw = blockDim.x >> 5;
-  for (int i = threadIdx.x >> 5; i < n; i += nw) {
-    const T* row = d.kinv + (size_t)i * n;
-    T acc = T(0);
-#pragma unroll 4
-    for (int j = lane; j < n; j += 32) acc = fma(row[j], g[j], acc);
-    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-    if (lane == 0) d.U[i] = acc;
-  }
-}
-
 }  // namespace dev
 }  // namespace igamg

@@ -885,6 +885,97 @@ int build_patches(int p, const Level1D& L, const igamg_sizes& s, PatchTables& pt
 
 }  // namespace
 
+bool patch_grids(int p, const igamg_sizes& s, const PatchTables& pt, bool by_row, int entry_bytes, PatchGrids& G) {
+  G = PatchGrids();
+  const int LW = p == 2 ? 32 : 64, TC = 2 * p + 1, NC = 2 * TC + 1;
+  if (pt.maxl > LW || (int)pt.pos.size() != pt.n_patches) return false;
+  PatchGrids out;
+  std::map<int, int> wcls;                                     // class (or -1 - class8) -> entry of wspec
+  out.colour.resize(pt.n_colours);
+  const int n = s.n, q = p - 1, np1 = p + 1, lo = p + 1, hi = n - 2, ni = n + p - 2, lq = n + p - 2;
+  const int nu = (int)(s.n_ux + s.n_uy);
+  // staged arrays (kernels_patch.cuh, PatchShape): extents, offsets and margin
+  const int W = 2 * p, A1 = 2 * p + 1, B1 = 2 * p, C1 = 2 * q + 1, UY = A1 * W, PX = 2 * UY, PY = PX + W * W;
+  const int REG = PY + W * W, MARGIN = (p + 1) * W;
+  for (int c = 0; c < pt.n_colours; ++c) {
+    PatchGrid& g = out.colour[c];
+    const int ca = c % np1, cb = c / np1;
+    g.a0 = lo + ((ca - lo) % np1 + np1) % np1;
+    g.b0 = lo + ((cb - lo) % np1 + np1) % np1;
+    g.gfirst = (int)out.gcls.size();
+    g.wfirst = (int)out.wdesc.size() / 4;
+    const int first = pt.colour_off[c], count = pt.colour_off[c + 1] - first;
+    for (int i = first; i < first + count; ++i) {
+      const int a = pt.pos[i] & 0xffff, b = pt.pos[i] >> 16;
+      const bool is8 = i - first < pt.n8[c];
+      const int* pd = &pt.dofs[(size_t)i * pt.maxl];
+      if (a >= lo && a <= hi && b >= lo && b <= hi) {
+        if (!is8) return false;
+        if (b == g.b0) ++g.na;                                 // the first row of positions sets na
+        const int j = b == g.b0 ? 0 : (g.na ? g.n8 / g.na : -1), k8 = b == g.b0 ? g.n8 : (g.na ? g.n8 % g.na : 0);
+        if (a != g.a0 + k8 * np1 || b != g.b0 + j * np1) return false;
+        const int want[8] = {(int)gid(s, 0, a, b - 1), (int)gid(s, 0, a, b), (int)gid(s, 1, a - 1, b), (int)gid(s, 1, a, b),
+                             (int)gid(s, 2, a - 1, b - 1), (int)gid(s, 2, a, b - 1), (int)gid(s, 2, a - 1, b), (int)gid(s, 2, a, b)};
+        for (int k = 0; k < 8; ++k) if (pd[k] != want[k]) return false;
+        out.gcls.push_back(pt.cls[i]);
+        ++g.n8;
+        continue;
+      }
+      ++g.nwall;
+      const int nl = is8 ? 8 : pt.nloc[pt.cls[i]];
+      int nv = 0;
+      for (int r = 0; r < LW; ++r) {
+        if (r >= nl) { out.wrow.insert(out.wrow.end(), {0, 0, 0, 0}); continue; }
+        if (pd[r] < 0 || pd[r] >= (int)s.n_total - 1) return false;
+        if (pd[r] < nu && r != nv) return false;               // velocity rows first
+        nv += pd[r] < nu;
+        const Dof D = decode(s, pd[r]);
+        const int dx = D.x - a, dy = D.y - b;
+        // [from, to] clipped to the index range [first, last] must lie in [ctr - p, ctr + p - 1 + own]
+        auto in = [&](int from, int to, int fst, int last, int ctr, int own) {
+          from = std::max(from, fst);
+          to = std::min(to, last);
+          return from > to || (from >= ctr - p && to <= ctr + p - 1 + own);
+        };
+        auto fits = [&](int off, int len, int across) {        // a box from entry off of the arrays
+          return off >= -MARGIN && off + (len - 1) * W + across - 1 < REG + MARGIN;
+        };
+        bool ok;
+        int oA, oB, oE = 0;                                    // where the row's boxes start
+        if (D.blk == 0) {
+          oA = dx * W + dy + 1; oB = PX + dx * W + dy + 1; oE = UY + (dy + 1) * W + dx;
+          ok = in(D.x - p, D.x + p, 1, ni, a, 1) && in(D.y - q, D.y + q, 0, lq, b, 0) && in(D.x - p, D.x + q, 0, lq, a, 0) &&
+               in(D.y - q, D.y + p, 1, ni, b, 1);
+        } else if (D.blk == 1) {
+          oA = UY + dy * W + dx + 1; oB = PY + dy * W + dx + 1; oE = (dx + 1) * W + dy;
+          ok = in(D.y - p, D.y + p, 1, ni, b, 1) && in(D.x - q, D.x + q, 0, lq, a, 0) && in(D.y - p, D.y + q, 0, lq, b, 0) &&
+               in(D.x - q, D.x + p, 1, ni, a, 1);
+        } else {
+          oA = (dx + 1) * W + dy + 1; oB = UY + (dy + 1) * W + dx + 1;
+          ok = in(D.x - q, D.x + p, 1, ni, a, 1) && in(D.y - q, D.y + q, 0, lq, b, 0) && in(D.y - q, D.y + p, 1, ni, b, 1) &&
+               in(D.x - q, D.x + q, 0, lq, a, 0);
+        }
+        if (!ok || !fits(oA, A1, C1) || !fits(oB, B1, C1) || (D.blk != 2 && !fits(oE, W, W))) return false;
+        const int cl = cls1(D.x, D.blk == 0 ? n + p - 1 : n + p - 2, TC) * NC + cls1(D.y, D.blk == 1 ? n + p - 1 : n + p - 2, TC);
+        out.wrow.insert(out.wrow.end(), {pd[r], (int)((unsigned)(oA & 0xffff) | ((unsigned)oB << 16)), oE,
+                                         by_row ? pd[r] : D.blk * NC * NC + cl});
+      }
+      if (is8 && nv != 4) return false;
+      const int key = is8 ? -1 - pt.cls[i] : pt.cls[i], rows = nl | (nv << 8);
+      auto it = wcls.find(key);
+      if (it == wcls.end()) {
+        it = wcls.emplace(key, (int)out.wspec.size() / 4).first;
+        out.wspec.insert(out.wspec.end(), {key, out.winv16, rows, 0});
+        out.winv16 += (nl * ((nl + 1) | 1) * entry_bytes + 15) / 16;   // wall_ld(nl) entries per row
+      }
+      out.wdesc.insert(out.wdesc.end(), {a | (b << 16), out.wspec[(size_t)4 * it->second + 1], rows, 0});
+    }
+    if (g.na > 0 && g.n8 % g.na) return false;
+  }
+  G = std::move(out);
+  return true;
+}
+
 void build_row_slots(PatchTables& pt) {
   const int maxl = pt.maxl;
   // 128-slot blocks where the patches allow (twice the blocks: a colour spreads more evenly

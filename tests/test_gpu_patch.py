@@ -1,0 +1,95 @@
+"""The staged patch kernels (shared-memory neighbourhoods; integer limbs for FP64) against the
+row-by-row colour kernels, at the sizes where their index rules change: meshes so small that
+every patch touches a wall or two, the first mesh with interior patches, ragged counts of
+patches per warp; every operator form; value ranges near the ends of FP64.
+
+Tolerances: a sweep is a few dozen sums of products per unknown and colour; both sides round
+each at 2^-53 or better of its largest term, and a colour's correction passes through at most
+(p+1)^2 later colours: 1e-12 (FP64) and 5e-5 (FP32, the same with 2^-24) of the largest unknown.
+"""
+import numpy as np
+import pytest
+
+from paper_1705_09282_gb300 import inputs
+
+pytestmark = pytest.mark.gpu
+
+
+def _torch():
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    return torch
+
+
+def _pair(monkeypatch, *args, **kw):
+    from paper_1705_09282_gb300.solver import Solver
+    S1 = Solver(*args, **kw)
+    monkeypatch.setenv("IGAMG_SWEEP_FORM", "lanes1")
+    monkeypatch.setenv("IGAMG_FUSED_LEVELS", "-1")
+    S0 = Solver(*args, **kw)
+    monkeypatch.delenv("IGAMG_SWEEP_FORM")
+    monkeypatch.delenv("IGAMG_FUSED_LEVELS")
+    return S0, S1
+
+
+@pytest.mark.parametrize("p", [2, 3])
+@pytest.mark.parametrize("n", [4, 6, 8, 10, 14, 22, 46])
+@pytest.mark.parametrize("kind", ["stokes", "oseen", "annulus", "fp32"])
+def test_staged_sweeps_equal_row_kernels(p, n, kind, monkeypatch):
+    torch = _torch()
+    from paper_1705_09282_gb300 import _lib
+    kw = {}
+    if kind == "oseen":
+        kw["beta"] = inputs.oseen_advection(p, n, 0.5)
+    elif kind == "annulus":
+        kw["geometry"] = _lib.IGAMG_GEOM_QUARTER_ANNULUS
+    elif kind == "fp32":
+        kw["precision"] = _lib.IGAMG_FP32_IR
+    S0, S1 = _pair(monkeypatch, p, n, 2, 10.0, 0.5, **kw)
+    nd = S0.ndof()
+    dt = torch.float32 if kind == "fp32" else torch.float64
+    U = torch.tensor(inputs.random_vector(nd, seed=n), device="cuda").to(dt)
+    F = torch.tensor(inputs.random_vector(nd, seed=n + 1), device="cuda").to(dt)
+    U0, U1 = U.clone(), U.clone()
+    for S, V in ((S0, U0), (S1, U1)):
+        (S.smooth32 if kind == "fp32" else S.smooth)(V, F, sweeps=1)
+    tol = 5e-5 if kind == "fp32" else 1e-12
+    assert float((U0 - U1).abs().max()) <= tol * float(U0.abs().max())
+    S0.close()
+    S1.close()
+
+
+@pytest.mark.parametrize("scale", [2.0 ** -600, 2.0 ** 600, 0.0])
+def test_staged_sweep_at_extreme_scales(scale, monkeypatch):
+    # the sweep is linear in (U, F): a power of two changes exponents only
+    torch = _torch()
+    from paper_1705_09282_gb300.solver import Solver
+    S = Solver(2, 16, 2, 1.0, 1.0)
+    nd = S.ndof()
+    U = torch.tensor(inputs.random_vector(nd, seed=3), device="cuda")
+    F = torch.tensor(inputs.random_vector(nd, seed=4), device="cuda")
+    V, W = U.clone(), U * scale
+    S.smooth(V, F, sweeps=2)
+    S.smooth(W, F * scale, sweeps=2)
+    assert torch.equal(W, V * scale)
+    S.close()
+
+
+@pytest.mark.parametrize("bad", [float("nan"), float("inf"), -float("inf")])
+@pytest.mark.parametrize("where", ["U", "F"])
+def test_staged_sweep_spreads_nonfinite_values_as_the_row_kernel_does(bad, where, monkeypatch):
+    torch = _torch()
+    S0, S1 = _pair(monkeypatch, 2, 32, 2, 1.0, 1.0)
+    nd = S0.ndof()
+    g = nd // 3
+    out = []
+    for S in (S0, S1):
+        U = torch.tensor(inputs.random_vector(nd, seed=5), device="cuda")
+        F = torch.tensor(inputs.random_vector(nd, seed=6), device="cuda")
+        (U if where == "U" else F)[g] = bad
+        S.smooth(U, F, sweeps=1)
+        out.append(torch.isfinite(U))
+        S.close()
+    assert not out[1][g] if where == "F" else True
+    assert torch.equal(out[0], out[1])
