@@ -24,6 +24,7 @@
 #include "igamg3d.h"
 #include "igamg_internal.h"
 #include "kernels3d.cuh"
+#include "kernels_patch3.cuh"
 #include "krylov.h"
 
 using namespace igamg;
@@ -193,6 +194,7 @@ template <typename T>
 struct Lev3T {
   LevelTab3<T> L{};
   T *cinv = nullptr, *cinv8 = nullptr, *cinv_all = nullptr;
+  PatchTab3<T> X{};                 // staged patch solves
   Xfer<T> tp{}, tq{};
   T *U = nullptr, *F = nullptr, *R = nullptr;
 };
@@ -215,6 +217,8 @@ struct Lev3Common {
   int *slot_g = nullptr, *slot_c = nullptr;
   unsigned* slot_kb = nullptr;
   long long* cinv_off = nullptr;
+  bool staged = false;              // staged patch solves (kernels_patch3.cuh)
+  std::vector<ColourGrid3> grids;
   double *dcoef = nullptr, *inv_dcoef = nullptr;
 };
 
@@ -297,6 +301,85 @@ template <typename T> Typed3<T>& typed(igamg3d_handle* h);
 template <> Typed3<double>& typed<double>(igamg3d_handle* h) { return h->d; }
 template <> Typed3<float>& typed<float>(igamg3d_handle* h) { return h->f; }
 
+// The staged patch kernels' tables of level l, made on the device from the uploaded ones.  Sets
+// lc.staged if the level suits those kernels.
+template <int P, typename T>
+int build_patch_tab3(igamg3d_handle* h, int l, Lev3T<T>& tl) {
+  using E = limb_t<T>;
+  auto& hl = h->host.lev[l];
+  auto& lc = h->lc[l];
+  const LevelTab3<T>& L = tl.L;
+  PatchTab3<T>& X = tl.X;
+  int nrec[4], total = 0, rc;
+  for (int k = 0; k < 4; ++k) {
+    nrec[k] = (int)(hl.st.rec[k].size() / Rec3<P>::RU);
+    X.koff[k] = total;
+    total += nrec[k];
+  }
+  PatchGrids3 G;
+  X.by_row = L.srow != nullptr;
+  if (!patch_grids3(P, hl.sz, hl.pt, hl.st, X.koff, X.by_row, (int)sizeof(E), G)) { lc.staged = false; return IGAMG_OK; }
+  lc.staged = true;
+  lc.grids.clear();
+  for (const PatchGrid3& g : G.colour) {
+    ColourGrid3 c;
+    c.f = g.f; c.n8 = g.n8; c.gfirst = g.gfirst; c.wfirst = g.wfirst; c.nwall = g.nwall;
+    for (int a = 0; a < 3; ++a) { c.o[a] = g.o[a]; c.s[a] = g.s[a]; c.cnt[a] = std::max(g.cnt[a], 1); }
+    for (int r = 0; r < 8; ++r) {
+      c.kind[r] = g.kind[r]; c.d[r] = g.d[r];
+      c.oA[r] = g.oA[r]; c.oB[r] = g.oB[r]; c.oC[r] = g.oC[r]; c.oE[r] = g.oE[r];
+    }
+    lc.grids.push_back(c);
+  }
+  X.maxl = 8;
+  for (size_t i = 0; i < G.wspec.size(); i += 4) X.maxl = std::max(X.maxl, G.wspec[i + 2] & 0xffff);
+  int *gcls, *wdesc, *wrow, *wspec;
+  if ((rc = upload_as(h, &gcls, G.gcls)) || (rc = upload_as(h, &wdesc, G.wdesc)) || (rc = upload_as(h, &wrow, G.wrow)) ||
+      (rc = upload_as(h, &wspec, G.wspec)))
+    return rc;
+  X.gcls = gcls;
+  X.wdesc = reinterpret_cast<const int4*>(wdesc);
+  X.wrow = reinterpret_cast<const int4*>(wrow);
+  constexpr int NR = rec3_len<P, T>();
+  E *rec, *inv8, *winv;
+  if (L.srow) {
+    const int n = L.n_total - 1;
+    if ((rc = dmalloc(h, (void**)&rec, (size_t)n * NR * sizeof(E)))) return rc;
+    k_patch_records3<P, T><<<nblk(n), kBlock, 0, h->stream>>>(n, -1, L.n_u, L.srow, rec);
+  } else {
+    const T* src[4] = {L.rc0, L.rc1, L.rc2, L.rc3};
+    if ((rc = dmalloc(h, (void**)&rec, (size_t)total * NR * sizeof(E)))) return rc;
+    for (int k = 0; k < 4; ++k)
+      if (nrec[k] > 0)
+        k_patch_records3<P, T><<<nblk(nrec[k]), kBlock, 0, h->stream>>>(nrec[k], k, 0, src[k], rec + (size_t)X.koff[k] * NR);
+  }
+  X.rec = rec;
+  if (L.sext) {
+    const int n = 2 * L.n_uc;
+    E* ext;
+    if ((rc = dmalloc(h, (void**)&ext, (size_t)n * ext3_rec_len<P, T>() * sizeof(E)))) return rc;
+    k_patch_ext3<P, T><<<nblk(n), kBlock, 0, h->stream>>>(n, L.n_uc, L.sext, ext);
+    X.ext = ext;
+  }
+  const int n8 = hl.pt.n_cls8, nw = (int)G.wspec.size() / 4;
+  if ((rc = dmalloc(h, (void**)&inv8, (size_t)std::max(n8, 1) * 8 * inv8_ld<T>() * sizeof(E))) ||
+      (rc = dmalloc(h, (void**)&winv, (size_t)std::max(G.winv16, 1) * 16)))
+    return rc;
+  if (n8 > 0) k_patch_inv8_3<T><<<nblk(n8 * 8), kBlock, 0, h->stream>>>(n8, hl.pt.n_cls, lc.cinv_off, tl.cinv_all, inv8);
+  if (nw > 0) k_patch_winv3<T><<<nw, 64, 0, h->stream>>>(reinterpret_cast<const int4*>(wspec), lc.cinv_off, tl.cinv_all, winv);
+  X.inv8 = inv8;
+  X.winv = winv;
+  return launch_check();
+}
+
+// Levels that suit the staged patch kernels use them (measured faster on every level; figures in
+// kernels_patch3.cuh); IGAMG_SWEEP_FORM=rows, read at creation, and the row kernels' own switches
+// keep the row kernels.
+bool staged_on() {
+  const char* e = std::getenv("IGAMG_SWEEP_FORM");
+  return !(e && std::strcmp(e, "rows") == 0) && row_parallel() && !std::getenv("IGAMG_ROW_SPLIT");
+}
+
 template <typename T>
 int upload_typed(igamg3d_handle* h, Typed3<T>& ty) {
   const int L = (int)h->host.lev.size();
@@ -332,6 +415,8 @@ int upload_typed(igamg3d_handle* h, Typed3<T>& ty) {
       if (hl.rows.empty() && ((rc = upload_as(h, &tl.cinv, hl.pt.cinv)) || (rc = upload_as(h, &tl.cinv8, hl.pt.cinv8))))
         return rc;
       if ((rc = upload_as(h, &tl.cinv_all, hl.pt.cinv_all))) return rc;
+      if (staged_on() && (rc = h->prob.p == 2 ? build_patch_tab3<2, T>(h, l, tl) : build_patch_tab3<3, T>(h, l, tl)))
+        return rc;
       auto up = [&](const Transfer1D& t, Xfer<T>& x) -> int {
         x.nf = t.nf; x.nc = t.nc;
         int r;
@@ -361,10 +446,47 @@ int do_residual(igamg3d_handle* h, int l, const T* U, const T* F, T* R, double* 
   return launch_check();
 }
 
+// Most blocks of a colour launch whose records are fetched ahead of the dependency wait (PRE of
+// k_patch_colour3).  Measured at p = 2, FP64, per colour: 32^3 (about 500 blocks) 10.3 us ahead, 10.4
+// in place, Oseen records 12.2 and 13.9; 64^3 (3600 blocks) 52.7 and 40.1.
+constexpr int kPreBlocks = 1500;
+
+// One sweep of staged patch solves, one launch per colour, each allowed to fetch its tables while the
+// launch before it runs (programmatic dependent launch, as in the 2D path).
+template <int P, typename T>
+int do_smooth_staged(igamg3d_handle* h, int l, T* U, const T* F, cudaStream_t s) {
+  using S = PatchShape3<P>;
+  auto& lc = h->lc[l];
+  auto& tl = typed<T>(h).lev[l];
+  cudaLaunchConfig_t cfg = {};
+  cfg.blockDim = dim3(S::NT);
+  cfg.dynamicSmemBytes = patch3_smem<P, T>(tl.X.maxl);
+  cfg.stream = s;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  for (const ColourGrid3& C : lc.grids) {
+    const int nb = C.nwall + (C.n8 + S::PPB - 1) / S::PPB;
+    if (nb == 0) continue;
+    cfg.gridDim = dim3((unsigned)nb);
+    const bool pre = nb <= kPreBlocks;
+    cudaError_t e;
+    if (tl.X.ext) e = pre ? cudaLaunchKernelEx(&cfg, k_patch_colour3<P, T, true, true>, tl.L, tl.X, U, F, C)
+                          : cudaLaunchKernelEx(&cfg, k_patch_colour3<P, T, true, false>, tl.L, tl.X, U, F, C);
+    else e = pre ? cudaLaunchKernelEx(&cfg, k_patch_colour3<P, T, false, true>, tl.L, tl.X, U, F, C)
+                 : cudaLaunchKernelEx(&cfg, k_patch_colour3<P, T, false, false>, tl.L, tl.X, U, F, C);
+    if (e != cudaSuccess) { set_error(cudaGetErrorString(e)); return IGAMG_ECUDA; }
+  }
+  return IGAMG_OK;
+}
+
 template <typename T>
 int do_smooth(igamg3d_handle* h, int l, T* U, const T* F, cudaStream_t s) {
   auto& lc = h->lc[l];
   auto& tl = typed<T>(h).lev[l];
+  if (lc.staged) return h->prob.p == 2 ? do_smooth_staged<2, T>(h, l, U, F, s) : do_smooth_staged<3, T>(h, l, U, F, s);
   if ((row_parallel() || tl.L.srow) && lc.row_slots) {
     const int S = lc.row_slots;
     const int* sg = lc.slot_g; const int* sc = lc.slot_c; const unsigned* sk = lc.slot_kb;

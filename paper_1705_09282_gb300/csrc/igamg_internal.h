@@ -58,7 +58,7 @@ struct PatchTables {
   std::vector<double> cinv8;   // n_cls8 * 64: the same for 8-DOF patches, packed 8 x 8
   std::vector<int> colour_off; // n_colours + 1
   std::vector<int> n8;         // per colour: patches with 4+4 DOFs, stored first in the colour
-  std::vector<int> pos;         // 2D: per patch its streamfunction position a | b << 16
+  std::vector<int> pos;         // per patch its position: 2D a | b << 16, 3D i | j << 10 | k << 20
   std::vector<int> d2p_off;    // dof -> list of (patch * maxl + local row), CSR over dofs
   std::vector<int> d2p_idx;
   // Row-flat view for the row-parallel colour kernel: each colour is cut into blocks of
@@ -261,6 +261,28 @@ struct HierarchyHost3 {
   int geometry = 0;
   std::vector<double> quad_xyz, jt;
 };
+
+// The 3D counterpart of PatchGrid / PatchGrids (kernels_patch3.cuh): per colour the family f, the
+// interior patches at o[a] + i_a s[a], i_a < cnt[a] (axis 0 fastest), and what their eight local
+// rows are: kind, position relative to the patch (bit a: one less along axis a), offsets of the
+// boxes A, B, C and of the third box in the staged arrays.
+struct PatchGrid3 {
+  int f = 0, o[3] = {1, 1, 1}, s[3] = {1, 1, 1}, cnt[3] = {0, 0, 0}, n8 = 0, gfirst = 0, wfirst = 0, nwall = 0;
+  int kind[8] = {}, d[8] = {}, oA[8] = {}, oB[8] = {}, oC[8] = {}, oE[8] = {};
+};
+struct PatchGrids3 {
+  std::vector<PatchGrid3> colour;
+  std::vector<int> gcls;       // interior patches: 8-row class
+  std::vector<int> wdesc;      // 4 ints per other patch: position, offset of the inverse (16 bytes),
+                               // rows | velocity rows << 16, 0
+  std::vector<int> wrow;       // 4 ints per row, mr rows per patch (64 at p = 2, 192 at p = 3): the row,
+                               // offsets A | B << 16, C | third box << 16, record
+  std::vector<int> wspec;      // 4 ints per class of those: class in cinv_all, offset, rows, 0
+  int winv16 = 0;
+};
+// koff: first record of each row kind; checks as patch_grids.
+bool patch_grids3(int p, const Sizes3& s, const PatchTables& pt, const Stencils3& st, const int* koff, bool by_row,
+                  int entry_bytes, PatchGrids3& G);
 
 int build_hierarchy3(const igamg_problem& pr, HierarchyHost3& H, std::string& err);
 // the finest level's 1D factors and row records only (no patches, transfers, coarse inverse)

@@ -33,7 +33,7 @@
 // the launch's own indices, fetched first and before the wait for the previous kernel
 // (programmatic dependent launch), so a colour's chain is: wait, one fetch of U and F, arithmetic.
 // Measured per colour launch (graph replay; row kernels k_mult_colour -> these), FP64: p = 2
-// 8^2-64^2 5.0-5.4 -> 2.1-2.3 us, 128^2 5.4 -> 2.9, 256^2 8.1 -> 6.4; p = 3 10-10.5 -> 2.6-2.9,
+// 8^2-64^2 5.0-5.4 -> 2.1-2.3 us, 128^2 5.4 -> 2.9, 256^2 8.1 -> 6.3; p = 3 10-10.5 -> 2.6-2.9,
 // 256^2 11.1 -> 7.0; generalized Oseen 512^2 V-cycle 2908 -> 2109 us.  FP32 (same staging, FP32
 // arithmetic): p = 2 4.1 -> 1.4-1.9 us, p = 3 7.6 -> 1.3-1.7.
 #pragma once
@@ -48,10 +48,14 @@ struct PatchShape {
   static constexpr int A1 = 2 * P + 1, B1 = 2 * P, C1 = 2 * Q + 1;  // box extents (long, long, across)
   static constexpr int NA = A1 * C1, NB = B1 * C1, RU = NA + NB + 1;
   static constexpr int NUX = A1 * W, NP = W * W;
-  static constexpr int UY = NUX, PX = 2 * NUX, PY = PX + NP, REG = PY + NP;
+  // offsets of the arrays and of the next patch: chosen so that the two patches of a half-warp and
+  // their eight rows read from different banks (entries of 8 bytes, offsets mod 16)
+  static constexpr int UY = P == 2 ? 22 : 56, PX = P == 2 ? 48 : 112, PY = P == 2 ? 68 : 150, REG = P == 2 ? 88 : 196;
   static constexpr int NLOAD = 2 * NUX + NP;                   // distinct values
   static constexpr int MARGIN = (P + 1) * W;                   // on both sides of a wall patch's arrays
-  static constexpr int NREC = (RU + 2 + 3) / 4 * 4;            // entries per row record (limbs + exponents)
+  // a row record: box A, box B from entry RA on (FP64: then the exponents of both), the lambda
+  // coefficient at IL (FP64: then its exponent)
+  static constexpr int RA = (NA + 3) / 4 * 4, IL = RA + NB + 1, NREC = (IL + 2 + 3) / 4 * 4;
   static constexpr int NEXT = (W * W + 1 + 3) / 4 * 4;         // third box: limbs + exponent
   static constexpr int LW = P == 2 ? 32 : 64;                  // threads per wall patch (rows <= 21, 40)
 };
@@ -151,6 +155,22 @@ __device__ __forceinline__ void ld_entries(const E* __restrict__ p, E* r) {   //
   for (int i = 0; i < N; i += V) ld_table(p + i, r + i);
 }
 
+// The same where they are used, for the compiler to schedule.
+template <int N, typename E>
+__device__ __forceinline__ void ld_entries_lazy(const E* __restrict__ p, E* r) {
+  constexpr int V = 16 / sizeof(E);
+  static_assert(N % V == 0, "whole 16-byte loads");
+#pragma unroll
+  for (int i = 0; i < N; i += V) {
+    const int4 q = __ldg(reinterpret_cast<const int4*>(p + i));
+    if constexpr (V == 2) { r[i] = make_int2(q.x, q.y); r[i + 1] = make_int2(q.z, q.w); }
+    else {
+      r[i] = __int_as_float(q.x); r[i + 1] = __int_as_float(q.y);
+      r[i + 2] = __int_as_float(q.z); r[i + 3] = __int_as_float(q.w);
+    }
+  }
+}
+
 // Waits until the kernels before this one in the stream have finished and their results are
 // visible, then lets the next kernel of the stream start its own table loads.  Without the
 // launch attribute both are no-ops.
@@ -165,22 +185,30 @@ template <> struct Resid<double> { long long v; int a; };
 
 // R = F - (box A) - (box B) - (third box) - m lambda for one row whose boxes start at sA, sB, sE.
 // exA, exB, exE: exponents of the staged values in the three boxes; st: the row's record.
-template <int P, typename T, bool EXT>
+// PRE: in registers; else in global memory, read box by box (boxes begin on 16 bytes: RA).
+template <int P, typename T, bool EXT, bool PRE>
 __device__ __forceinline__ Resid<T> row_resid(const limb_t<T>* sA, const limb_t<T>* sB, const limb_t<T>* sE,
                                               const limb_t<T>* st, const limb_t<T>* __restrict__ se,
                                               bool is_p, int exA, int exB, int exE, T f, T lam) {
   using S = PatchShape<P>;
   if constexpr (sizeof(T) == 8) {
     Acc A, B;
+    {
+      limb_t<T> own[S::RA];
+      if constexpr (!PRE) ld_entries_lazy<S::RA>(st, own);
+      const limb_t<T>* k = PRE ? st : own;
 #pragma unroll
-    for (int d = 0; d < S::A1; ++d)
+      for (int j = 0; j < S::NA; ++j) A.mac(sA[(j / S::C1) * S::W + j % S::C1], k[j]);
+    }
+    int2 ec;
+    {
+      limb_t<T> own[S::NREC - S::RA];
+      if constexpr (!PRE) ld_entries_lazy<S::NREC - S::RA>(st + S::RA, own);
+      const limb_t<T>* k = PRE ? st + S::RA : own;
 #pragma unroll
-      for (int e = 0; e < S::C1; ++e) A.mac(sA[d * S::W + e], st[d * S::C1 + e]);
-#pragma unroll
-    for (int d = 0; d < S::B1; ++d)
-#pragma unroll
-      for (int e = 0; e < S::C1; ++e) B.mac(sB[d * S::W + e], st[S::NA + d * S::C1 + e]);
-    const int2 ec = st[S::RU];
+      for (int j = 0; j < S::NB; ++j) B.mac(sB[(j / S::C1) * S::W + j % S::C1], k[j]);
+      ec = k[S::NB];
+    }
     const int aA = exA + ec.x, aB = exB + ec.y, exF = exp_of(f);
     int a = max(max(aA, aB), max(exF, kExpFloor));
     long long sE_ = 0, sL = 0;
@@ -198,8 +226,8 @@ __device__ __forceinline__ Resid<T> row_resid(const limb_t<T>* sA, const limb_t<
     if (is_p && lam != 0.0) {                                  // (lam is the same for the whole grid)
       const int exL = max(exp_of(lam), kExpFloor);
       Acc Lm;
-      Lm.mac(to_limbs(lam, exL), st[S::RU - 1]);
-      aL = exL + st[S::RU + 1].x;
+      Lm.mac(to_limbs(lam, exL), st[S::IL]);
+      aL = exL + st[S::IL + 1].x;
       sL = Lm.sum();
       a = max(a, aL);
     }
@@ -214,19 +242,22 @@ __device__ __forceinline__ Resid<T> row_resid(const limb_t<T>* sA, const limb_t<
     return {r, a};
   } else {
     T a0 = T(0), a1 = T(0), b0 = T(0), b1 = T(0);
+    limb_t<T> own[PRE ? 4 : S::NREC];
+    if constexpr (!PRE) ld_entries_lazy<S::NREC>(st, own);
+    const limb_t<T>* k = PRE ? st : own;
 #pragma unroll
     for (int j = 0; j < S::NA; ++j) {
       const T v = sA[(j / S::C1) * S::W + j % S::C1];
-      if (j & 1) a1 = fma(st[j], v, a1);
-      else a0 = fma(st[j], v, a0);
+      if (j & 1) a1 = fma(k[j], v, a1);
+      else a0 = fma(k[j], v, a0);
     }
 #pragma unroll
     for (int j = 0; j < S::NB; ++j) {
       const T v = sB[(j / S::C1) * S::W + j % S::C1];
-      if (j & 1) b1 = fma(st[S::NA + j], v, b1);
-      else b0 = fma(st[S::NA + j], v, b0);
+      if (j & 1) b1 = fma(k[S::RA + j], v, b1);
+      else b0 = fma(k[S::RA + j], v, b0);
     }
-    if (is_p) b1 = fma(st[S::RU - 1], lam, b1);
+    if (is_p) b1 = fma(k[S::IL], lam, b1);
     if (EXT && !is_p) {
 #pragma unroll
       for (int j = 0; j < S::W * S::W; ++j) {
@@ -260,11 +291,12 @@ __device__ __forceinline__ int group_max8(int v) {
 // tables(): everything that does not depend on U or F, into registers (one memory round trip that
 // overlaps the previous kernel); solve(): the neighbourhood, the residual rows, the inverse.
 // All 32 lanes call together.
-template <int P, typename T, bool EXT>
+template <int P, typename T, bool EXT, bool PRE>
 struct Patch8 {
   using S = PatchShape<P>;
   using E = limb_t<T>;
-  E st[S::NREC], A[inv8_ld<T>()];
+  E st_[PRE ? S::NREC : 4], A[PRE ? inv8_ld<T>() : 4];
+  const E *st, *Ap;
   int a, b, g;
   bool active;
 
@@ -283,8 +315,12 @@ struct Patch8 {
     const int k = X.by_row ? g
                            : (is_p ? 2 : (is_y ? 1 : 0)) * NC * NC +
                                  cls1d<P>(ix, is_p || is_y ? L.lastq : L.lastp) * NC + cls1d<P>(iy, is_y ? L.lastp : L.lastq);
-    ld_entries<S::NREC>(X.rec + (size_t)k * S::NREC, st);
-    ld_entries<inv8_ld<T>()>(X.inv8 + ((size_t)icls * 8 + row) * inv8_ld<T>(), A);
+    st = X.rec + (size_t)k * S::NREC;
+    Ap = X.inv8 + ((size_t)icls * 8 + row) * inv8_ld<T>();
+    if constexpr (PRE) {
+      ld_entries<S::NREC>(st, st_);
+      ld_entries<inv8_ld<T>()>(Ap, A);
+    }
   }
 
   __device__ __forceinline__ void solve(const LevelTab<T>& L, const PatchTab<T>& X, T* U, const T* F, int lane, E* sm) {
@@ -341,13 +377,21 @@ struct Patch8 {
         reg[S::PY + c * S::W + d] = v;
       }
     }
+    if constexpr (sizeof(T) == 4) {                            // pressure rows read the gap after UX times zero
+#pragma unroll
+      for (int k = S::NUX; k < S::UY; k += 8)
+        if (k + row < S::UY) reg[k + row] = T(0);
+    }
     __syncwarp();
     const E* sA = reg + (is_p ? o * S::W + o2 : (is_y ? S::UY + o : o));
     const E* sB = reg + (is_p ? S::UY + o2 * S::W + o : (is_y ? S::PY + o : S::PX + o));
     const E* sE = reg + (is_y ? o * S::W : S::UY + o * S::W);
     const E* se = EXT ? X.ext + (size_t)(is_p ? 0 : g) * S::NEXT : nullptr;
-    const Resid<T> r = row_resid<P, T, EXT>(sA, sB, sE, st, se, is_p, eu, is_p ? eu : ep, eu, f, lam);
+    const Resid<T> r = row_resid<P, T, EXT, PRE>(sA, sB, sE, PRE ? st_ : st, se, is_p, eu, is_p ? eu : ep, eu, f, lam);
     __syncwarp();
+    E A_[PRE ? 4 : inv8_ld<T>()];
+    if constexpr (!PRE) ld_entries_lazy<inv8_ld<T>()>(Ap, A_);
+    const E* A = PRE ? this->A : A_;
     if constexpr (sizeof(T) == 8) {
       const int er = resid_exp(r);
       int eg = max(er, __shfl_xor_sync(0xffffffffu, er, 1));
@@ -398,11 +442,11 @@ __host__ __device__ constexpr int group_entries(int maxl) {
 }
 
 // ---- the other patches (on or near a wall, up to LW rows): LW threads each, thread = row ----------
-template <int P, typename T, bool EXT>
+template <int P, typename T, bool EXT, bool PRE>
 struct PatchWall {
   using S = PatchShape<P>;
   using E = limb_t<T>;
-  E st[S::NREC];
+  E st_[PRE ? S::NREC : 4];
   int4 D, R;                        // D: a | b << 16, offset of the inverse (16 B), rows | velocity rows << 8
                                     // R: row, offset of box A | of box B << 16, of the third box, record
 
@@ -418,7 +462,7 @@ struct PatchWall {
     for (int i = t; i < n16; i += S::LW)
       asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst + 16 * i), "l"(src + 16 * (size_t)i) : "memory");
     asm volatile("cp.async.commit_group;" ::: "memory");
-    ld_entries<S::NREC>(X.rec + (size_t)R.w * S::NREC, st);    // threads past the last row: record 0
+    if constexpr (PRE) ld_entries<S::NREC>(X.rec + (size_t)R.w * S::NREC, st_);   // threads past the last row: record 0
   }
 
   __device__ __forceinline__ void solve(const LevelTab<T>& L, const PatchTab<T>& X, T* U, const T* F, int t, E* sm) {
@@ -464,7 +508,9 @@ struct PatchWall {
         bad = red[4] | red[5];
       }
     } else {
-      for (int i = t; i < S::MARGIN; i += S::LW) { sm[i] = T(0); reg[S::REG + i] = T(0); }
+      // what rows read with zero coefficients must be finite: the margins and the gaps
+      for (int i = t; i < 2 * S::MARGIN + S::REG; i += S::LW) sm[i] = T(0);
+      wall_sync<S::LW>();
     }
 #pragma unroll
     for (int k = 0; k < K; ++k) {
@@ -473,9 +519,10 @@ struct PatchWall {
       E w;
       if constexpr (sizeof(T) == 8) w = to_limbs(v[k], e >= 2 * S::NUX ? ep : eu);
       else w = v[k];
-      reg[e] = w;                                              // UX, UY and PX follow one another
+      const int e1 = e - (e >= 2 * S::NUX ? 2 * S::NUX : (e >= S::NUX ? S::NUX : 0));
+      reg[e1 + (e >= 2 * S::NUX ? S::PX : (e >= S::NUX ? S::UY : 0))] = w;
       if (e >= 2 * S::NUX) {
-        const int e1 = e - 2 * S::NUX, d = e1 / S::W;
+        const int d = e1 / S::W;
         reg[S::PY + (e1 - d * S::W) * S::W + d] = w;
       }
     }
@@ -483,7 +530,8 @@ struct PatchWall {
     const E* sA = reg + (short)(R.y & 0xffff);
     const E* sB = reg + (R.y >> 16);
     const E* se = EXT ? X.ext + (size_t)(is_p || !has ? 0 : g) * S::NEXT : nullptr;
-    const Resid<T> r = row_resid<P, T, EXT>(sA, sB, reg + R.z, st, se, is_p, eu, is_p ? eu : ep, eu, f, lam);
+    const Resid<T> r = row_resid<P, T, EXT, PRE>(sA, sB, reg + R.z, PRE ? st_ : X.rec + (size_t)R.w * S::NREC, se, is_p, eu,
+                                                 is_p ? eu : ep, eu, f, lam);
     asm volatile("cp.async.wait_all;" ::: "memory");
     const int ld = wall_ld(nl);
     const E* Ak = inv + (has ? t : 0) * ld;
@@ -525,19 +573,19 @@ struct PatchWall {
 // Group w of LW threads of one colour's work: the wall patches first (their chains are the
 // longest), then the interior patches, four to a warp along x.  WAIT: the kernel's dependency
 // wait stands between the table loads and the solve.
-template <int P, typename T, bool EXT, bool WAIT>
+template <int P, typename T, bool EXT, bool PRE, bool WAIT>
 __device__ __forceinline__ void colour_group(const LevelTab<T>& L, const PatchTab<T>& X, T* U, const T* F,
                                              const ColourGrid& C, int w, int t, limb_t<T>* sm) {
   using S = PatchShape<P>;
   if (w < C.nwall) {
-    PatchWall<P, T, EXT> W;
+    PatchWall<P, T, EXT, PRE> W;
     W.tables(X, C.wfirst + w, t, sm);
     if (WAIT) dependency_wait();
     W.solve(L, X, U, F, t, sm);
   } else {
     const int wp = (w - C.nwall) * (S::LW / 32) + (t >> 5);
     if (wp >= C.n8 / max(C.na, 1) * ((C.na + 3) >> 2)) return;
-    Patch8<P, T, EXT> I;
+    Patch8<P, T, EXT, PRE> I;
     I.tables(L, X, C, wp, t & 31);
     if (WAIT) dependency_wait();
     I.solve(L, X, U, F, t & 31, sm + (t >> 5) * 4 * S::REG);
@@ -549,7 +597,9 @@ __host__ __device__ inline int colour_groups(const ColourGrid& C) {
   return C.nwall + (C.n8 ? (C.n8 / C.na * ((C.na + 3) >> 2) + wpg - 1) / wpg : 0);
 }
 
-// One colour of the sweep.  Threads per block: 64 (two groups at p = 2, one at p = 3).
+// One colour of the sweep.  Threads per block: 64 (two groups at p = 2, one at p = 3).  The records
+// are fetched into registers before the dependency wait: reading them in place instead (twice the
+// warps per SM) measured 2.75 against 2.2 us on 64^2, 6.4 against 6.5 on 256^2 (p = 2).
 template <int P, typename T, bool EXT>
 __global__ void __launch_bounds__(64) k_patch_colour(const __grid_constant__ LevelTab<T> L, const __grid_constant__ PatchTab<T> X,
                                                      T* U, const T* F, const ColourGrid C, int ngroups, int smg) {
@@ -557,7 +607,7 @@ __global__ void __launch_bounds__(64) k_patch_colour(const __grid_constant__ Lev
   constexpr int LW = PatchShape<P>::LW;
   const int gib = threadIdx.x / LW, w = blockIdx.x * (64 / LW) + gib;
   if (w >= ngroups) return;
-  colour_group<P, T, EXT, true>(L, X, U, F, C, w, threadIdx.x % LW, reinterpret_cast<limb_t<T>*>(smem_raw) + gib * smg);
+  colour_group<P, T, EXT, true, true>(L, X, U, F, C, w, threadIdx.x % LW, reinterpret_cast<limb_t<T>*>(smem_raw) + gib * smg);
 }
 
 // ---- building the tables (once, at creation) ---------------------------------------------------
@@ -596,16 +646,17 @@ __global__ void k_patch_records(int n, int kind, int n_ux, int n_uy, const T* __
     for (int j = 0; j < S::NB; ++j) sb += fabs(s[S::NA + j]);
     const int ea = sum_exp(sa), eb = sum_exp(sb), el = sum_exp(fabs(s[S::RU - 1]));
     for (int j = 0; j < S::NA; ++j) d[j] = coef_limbs(s[box_src<P>(k, false, j)], ea);
-    for (int j = 0; j < S::NB; ++j) d[S::NA + j] = coef_limbs(s[box_src<P>(k, true, j)], eb);
-    d[S::RU - 1] = coef_limbs(s[S::RU - 1], el);
-    d[S::RU] = make_int2(ea, eb);
-    d[S::RU + 1] = make_int2(el, 0);
-    for (int j = S::RU + 2; j < S::NREC; ++j) d[j] = make_int2(0, 0);
+    for (int j = S::NA; j < S::RA; ++j) d[j] = make_int2(0, 0);
+    for (int j = 0; j < S::NB; ++j) d[S::RA + j] = coef_limbs(s[box_src<P>(k, true, j)], eb);
+    d[S::RA + S::NB] = make_int2(ea, eb);
+    d[S::IL] = coef_limbs(s[S::RU - 1], el);
+    d[S::IL + 1] = make_int2(el, 0);
+    for (int j = S::IL + 2; j < S::NREC; ++j) d[j] = make_int2(0, 0);
   } else {
     for (int j = 0; j < S::NA; ++j) d[j] = s[box_src<P>(k, false, j)];
-    for (int j = 0; j < S::NB; ++j) d[S::NA + j] = s[box_src<P>(k, true, j)];
-    d[S::RU - 1] = s[S::RU - 1];
-    for (int j = S::RU; j < S::NREC; ++j) d[j] = T(0);
+    for (int j = S::NA; j < S::NREC; ++j) d[j] = T(0);
+    for (int j = 0; j < S::NB; ++j) d[S::RA + j] = s[box_src<P>(k, true, j)];
+    d[S::IL] = s[S::RU - 1];
   }
 }
 
@@ -712,7 +763,7 @@ __global__ void __launch_bounds__(128) k_mix_colour(const __grid_constant__ MixA
     if (w >= colour_groups<P>(C)) return;
     const LevelTab<T> L = d.L;
     const PatchTab<T> X = d.X;
-    colour_group<P, T, EXT, false>(L, X, d.U, d.F, C, w, threadIdx.x % LW,
+    colour_group<P, T, EXT, false, false>(L, X, d.U, d.F, C, w, threadIdx.x % LW,
                                    reinterpret_cast<limb_t<T>*>(smem_raw) + gib * smg);
     return;
   }

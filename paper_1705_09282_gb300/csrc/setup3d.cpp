@@ -238,12 +238,14 @@ int build_patches3(int p, const Level1D& L, const Sizes3& s, PatchTables& pt, st
   pt.n_patches = (int)all.size(); pt.maxl = maxl; pt.n_colours = 3 * ncol_fam;
   pt.dofs.assign((size_t)pt.n_patches * maxl, -1);
   pt.cls.assign(pt.n_patches, 0);
+  if (n <= 1000) pt.pos.assign(pt.n_patches, 0);
   pt.colour_off.assign(pt.n_colours + 1, 0);
   std::map<std::tuple<int, int, int, int>, int> cmap8, cmapg;
   std::vector<int> rep8, repg;
   for (int i = 0; i < pt.n_patches; ++i) {
     auto& P_ = all[i];
     for (size_t k = 0; k < P_.dofs.size(); ++k) pt.dofs[(size_t)i * maxl + k] = P_.dofs[k];
+    if (!pt.pos.empty()) pt.pos[i] = P_.i[0] | (P_.i[1] << 10) | (P_.i[2] << 20);
     pt.colour_off[P_.colour + 1]++;
     bool is8 = P_.dofs.size() == 8;
     auto& cmap = is8 ? cmap8 : cmapg;
@@ -1235,6 +1237,164 @@ int host_patches3(const igamg_problem* prob, int level, int* colour, int* dofs, 
     std::copy(pt.dofs.begin(), pt.dofs.end(), dofs);
   }
   return IGAMG_OK;
+}
+
+
+bool patch_grids3(int p, const Sizes3& s, const PatchTables& pt, const Stencils3& st, const int* koff, bool by_row,
+                  int entry_bytes, PatchGrids3& G) {
+  G = PatchGrids3();
+  const int MR = p == 2 ? 64 : 192;
+  if (pt.maxl > MR || pt.pos.empty() || (int)pt.pos.size() != pt.n_patches) return false;
+  PatchGrids3 out;
+  out.colour.resize(pt.n_colours);
+  std::map<int, int> wcls;                                     // class -> entry of wspec
+  const int n = s.n, q = p - 1, ncol_fam = p * (p + 1) * (p + 1), T = 2 * p + 1, NC = 2 * T + 1;
+  // staged arrays (kernels_patch3.cuh, PatchShape3)
+  const int W = 2 * p, LS = W * W + (p == 2 ? 4 : 2), W3 = W * LS, A1 = 2 * p + 1, C1 = 2 * q + 1, LPR = p == 2 ? 4 : 8;
+  const int UC = A1 * LS, UF = 2 * UC, P1 = UF + W3, REGI = P1 + 2 * W3, REGW = REGI + W3, MARGIN = p * LS;
+  // offset of (start positions x0) in the array of component blk (3: pressure, ordered from axis c)
+  auto offset = [&](int f, const int* P, int blk, int c, const int* x0) {
+    const int c1 = (f + 1) % 3, base = blk < 3 ? (blk == f ? UF : (blk == c1 ? 0 : UC)) : P1 + (c == c1 ? 0 : (c == f ? 2 : 1)) * W3;
+    int off = 0;
+    for (int k = 0; k < 3; ++k) {
+      const int a = (c + k) % 3;
+      off += (k == 0 ? LS : (k == 1 ? W : 1)) * (x0[a] - (P[a] - (a == f ? q : p)));
+    }
+    return base + off;
+  };
+  // the row's boxes: component (array), axis order, and whether its positions fit
+  struct Off { int A, B, C, E; };
+  auto row_offsets = [&](int f, const int* P, const Dof3& D, bool wall, Off& o) -> bool {
+    o = Off{0, 0, 0, 0};
+    const int limit = (wall ? REGW : REGI) + (wall ? MARGIN : 0), low = wall ? -MARGIN : 0;
+    // box over component blk, long axis c with positions from .. to, across +-q
+    auto box = [&](int blk, int c, int from, int to, int* res, int slices) -> bool {
+      int x0[3];
+      for (int a = 0; a < 3; ++a) {
+        const bool own = blk < 3 && a == blk;
+        x0[a] = a == c ? D.i[a] + from : D.i[a] - q;
+        int lo = std::max(x0[a], own ? 1 : 0), hi = std::min(a == c ? D.i[a] + to : D.i[a] + q, own ? s.ni : s.nq - 1);
+        // the array holds: along f  P-q .. P+q (u_f: P-q .. P+p); else P-p .. P+p-1 (own axis: P+p)
+        const int alo = P[a] - (a == f ? q : p), ahi = P[a] + (a == f ? (blk == f ? p : q) : (own ? p : p - 1));
+        if (lo <= hi && (lo < alo || hi > ahi)) return false;
+      }
+      *res = offset(f, P, blk, c, x0);
+      return *res >= low && *res + (slices - 1) * LS + (C1 - 1) * W + C1 - 1 < limit;
+    };
+    bool ok;
+    if (D.blk < 3) {
+      ok = box(D.blk, D.blk, -p, p, &o.A, A1) && box(3, D.blk, -p, q, &o.B, 2 * p);
+      if (D.blk < 2) {                                         // third box of mapped domains: the other of u_x, u_y
+        const int ob = 1 - D.blk;
+        int x0[3], ok2 = 1;
+        for (int a = 0; a < 3; ++a) {
+          const bool own = a == ob;
+          x0[a] = a == 2 ? D.i[a] - q : (a == D.blk ? D.i[a] - p : D.i[a] - q);
+          const int end = a == 2 ? D.i[a] + q : (a == D.blk ? D.i[a] + q : D.i[a] + p);
+          const int lo = std::max(x0[a], own ? 1 : 0), hi = std::min(end, own ? s.ni : s.nq - 1);
+          const int alo = P[a] - (a == f ? q : p), ahi = P[a] + (a == f ? (ob == f ? p : q) : (own ? p : p - 1));
+          if (lo <= hi && (lo < alo || hi > ahi)) ok2 = 0;
+        }
+        o.E = offset(f, P, ob, ob, x0);
+        ok = ok && ok2 && o.E >= low && o.E + (W - 1) * LS + (W - 1) * W + W - 1 < limit;
+      }
+      // lane 0's extra slice of box A (p = 2) lies inside box A
+    } else {
+      ok = true;
+      int r[3];
+      for (int k = 0; k < 3; ++k) ok = ok && box(k, k, -q, p, &r[k], 2 * p);
+      o.A = r[0]; o.B = r[1]; o.C = r[2];
+      // p = 3: the lanes past the last slice of box A read one slice more (zero coefficients)
+      ok = ok && o.A + (std::min(LPR, A1) - 1) * LS + (C1 - 1) * W + C1 - 1 < limit;
+    }
+    return ok;
+  };
+  for (int c = 0; c < pt.n_colours; ++c) {
+    PatchGrid3& g = out.colour[c];
+    const int f = c / ncol_fam, cc = c % ncol_fam;
+    g.f = f;
+    int stride[3], lo[3], hi[3], cm[3];
+    for (int a = 0; a < 3; ++a) {
+      stride[a] = a == f ? p : p + 1;
+      lo[a] = a == f ? p : p + 1;
+      hi[a] = n - 2;
+    }
+    cm[0] = cc % stride[0]; cm[1] = cc / stride[0] % stride[1]; cm[2] = cc / (stride[0] * stride[1]);
+    int total = 1;
+    for (int a = 0; a < 3; ++a) {
+      g.s[a] = stride[a];
+      g.o[a] = lo[a] + ((cm[a] - lo[a]) % stride[a] + stride[a]) % stride[a];
+      g.cnt[a] = g.o[a] <= hi[a] ? (hi[a] - g.o[a]) / stride[a] + 1 : 0;
+      total *= g.cnt[a];
+    }
+    g.gfirst = (int)out.gcls.size();
+    g.wfirst = (int)out.wdesc.size() / 4;
+    for (int i = pt.colour_off[c]; i < pt.colour_off[c + 1]; ++i) {
+      const int P[3] = {pt.pos[i] & 1023, pt.pos[i] >> 10 & 1023, pt.pos[i] >> 20 & 1023};
+      const bool is8 = i - pt.colour_off[c] < pt.n8[c];
+      const int* pd = &pt.dofs[(size_t)i * pt.maxl];
+      bool inner = true;
+      for (int a = 0; a < 3; ++a) inner = inner && P[a] >= lo[a] && P[a] <= hi[a];
+      if (inner) {
+        const int k = g.n8, k2 = k / (g.cnt[0] * g.cnt[1]), k1 = k / g.cnt[0] % g.cnt[1], k0 = k % g.cnt[0];
+        if (!is8 || P[0] != g.o[0] + k0 * g.s[0] || P[1] != g.o[1] + k1 * g.s[1] || P[2] != g.o[2] + k2 * g.s[2]) return false;
+        for (int r = 0; r < 8; ++r) {
+          const Dof3 D = decode3(s, pd[r]);
+          int d = 0;
+          for (int a = 0; a < 3; ++a) {
+            const int m = P[a] - D.i[a];
+            if (m != 0 && m != 1) return false;
+            d |= m << a;
+          }
+          if (r < 4 ? D.blk == 3 : D.blk != 3) return false;
+          if (g.n8 == 0) {
+            Off o;
+            if (!row_offsets(f, P, D, false, o)) return false;
+            g.kind[r] = D.blk; g.d[r] = d;
+            g.oA[r] = o.A; g.oB[r] = o.B; g.oC[r] = o.C; g.oE[r] = o.E;
+          } else if (g.kind[r] != D.blk || g.d[r] != d) {
+            return false;
+          }
+        }
+        out.gcls.push_back(pt.cls[i]);
+        ++g.n8;
+        continue;
+      }
+      ++g.nwall;
+      const int cls = is8 ? pt.n_cls + pt.cls[i] : pt.cls[i], nl = is8 ? 8 : pt.nloc[pt.cls[i]];
+      int nv = 0;
+      for (int r = 0; r < MR; ++r) {
+        if (r >= nl) { out.wrow.insert(out.wrow.end(), {0, 0, 0, 0}); continue; }
+        if (pd[r] < 0 || pd[r] >= (int)s.n_total - 1) return false;
+        const Dof3 D = decode3(s, pd[r]);
+        if (D.blk < 3 && r != nv) return false;                // velocity rows first
+        nv += D.blk < 3;
+        Off o;
+        if (!row_offsets(f, P, D, true, o)) return false;
+        int rec = pd[r];
+        if (!by_row) {
+          const int lp = n + p - 1, lq = n + p - 2;
+          const int cl = (cls1(D.i[2], D.blk == 2 ? lp : lq, T) * NC + cls1(D.i[1], D.blk == 1 ? lp : lq, T)) * NC +
+                         cls1(D.i[0], D.blk == 0 ? lp : lq, T);
+          if (st.cmap[D.blk][cl] < 0) return false;
+          rec = koff[D.blk] + st.cmap[D.blk][cl];
+        }
+        auto pack = [](int a, int b) { return (int)((unsigned)(a & 0xffff) | ((unsigned)b << 16)); };
+        out.wrow.insert(out.wrow.end(), {pd[r], pack(o.A, o.B), pack(o.C, o.E), rec});
+      }
+      const int rows = nl | (nv << 16);
+      auto it = wcls.find(cls);
+      if (it == wcls.end()) {
+        it = wcls.emplace(cls, (int)out.wspec.size() / 4).first;
+        out.wspec.insert(out.wspec.end(), {cls, out.winv16, rows, 0});
+        out.winv16 += (nl * ((nl + 1) | 1) * entry_bytes + 15) / 16;
+      }
+      out.wdesc.insert(out.wdesc.end(), {pt.pos[i], out.wspec[(size_t)4 * it->second + 1], rows, 0});
+    }
+    if (g.n8 != total) return false;
+  }
+  G = std::move(out);
+  return true;
 }
 
 }  // namespace igamg
