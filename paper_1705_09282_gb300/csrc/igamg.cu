@@ -438,8 +438,8 @@ int do_smooth_staged(igamg_handle* h, int l, T* U, const T* F, cudaStream_t s) {
     const int ng = colour_groups<P>(C);
     if (ng == 0) continue;
     cfg.gridDim = dim3((unsigned)((ng + gpb - 1) / gpb));
-    const cudaError_t e = tl.X.ext ? cudaLaunchKernelEx(&cfg, k_patch_colour<P, T, true>, tl.L, tl.X, U, F, C, ng, smg)
-                                   : cudaLaunchKernelEx(&cfg, k_patch_colour<P, T, false>, tl.L, tl.X, U, F, C, ng, smg);
+    const cudaError_t e = tl.X.ext ? cudaLaunchKernelEx(&cfg, k_patch_colour<P, T, true>, tl.L, tl.X, U, F, C, ng, smg, 1)
+                                   : cudaLaunchKernelEx(&cfg, k_patch_colour<P, T, false>, tl.L, tl.X, U, F, C, ng, smg, 1);
     if (e != cudaSuccess) { g_err = cudaGetErrorString(e); return IGAMG_ECUDA; }
   }
   return IGAMG_OK;
@@ -1714,7 +1714,7 @@ int build_patch_tab(igamg_handle* h, int l, TypedLevel<T>& tl) {
     return rc;
   k_patch_inv8<T><<<nblk(n8 * 8), kBlock, 0, h->stream>>>(n8, tl.cinv8, inv8);
   if (nw > 0)
-    k_patch_winv<T><<<nw, S::LW, 0, h->stream>>>(lc.maxl, reinterpret_cast<const int4*>(wspec), tl.cinv, tl.cinv8, winv);
+    k_patch_winv<P, T><<<nw, S::LW, 0, h->stream>>>(lc.maxl, reinterpret_cast<const int4*>(wspec), tl.cinv, tl.cinv8, winv);
   X.inv8 = inv8;
   X.winv = winv;
   return launch_check();

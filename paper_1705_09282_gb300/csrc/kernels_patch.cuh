@@ -33,9 +33,9 @@
 // the launch's own indices, fetched first and before the wait for the previous kernel
 // (programmatic dependent launch), so a colour's chain is: wait, one fetch of U and F, arithmetic.
 // Measured per colour launch (graph replay; row kernels k_mult_colour -> these), FP64: p = 2
-// 8^2-64^2 5.0-5.4 -> 2.1-2.3 us, 128^2 5.4 -> 2.9, 256^2 8.1 -> 6.3; p = 3 10-10.5 -> 2.6-2.9,
-// 256^2 11.1 -> 7.0; generalized Oseen 512^2 V-cycle 2908 -> 2109 us.  FP32 (same staging, FP32
-// arithmetic): p = 2 4.1 -> 1.4-1.9 us, p = 3 7.6 -> 1.3-1.7.
+// 8^2-64^2 5.0-5.4 -> 1.9-2.1 us, 128^2 5.4 -> 2.5, 256^2 8.1 -> 5.0; p = 3 10-10.5 -> 2.5-2.7,
+// 256^2 11.1 -> 7.6; generalized Oseen 512^2 V-cycle 2908 -> 1966 us.  FP32 (same staging, FP32
+// arithmetic): p = 2 4.1 -> 1.5-1.8 us, p = 3 7.6 -> 1.3-1.6.
 #pragma once
 #include "kernels.cuh"
 
@@ -57,7 +57,10 @@ struct PatchShape {
   // coefficient at IL (FP64: then its exponent)
   static constexpr int RA = (NA + 3) / 4 * 4, IL = RA + NB + 1, NREC = (IL + 2 + 3) / 4 * 4;
   static constexpr int NEXT = (W * W + 1 + 3) / 4 * 4;         // third box: limbs + exponent
-  static constexpr int LW = P == 2 ? 32 : 64;                  // threads per wall patch (rows <= 21, 40)
+  static constexpr int LW = P == 2 ? 32 : 64;                  // threads per wall patch
+  // most velocity and pressure rows of a wall patch; rows of its inverse: MV velocity columns, MP
+  // pressure columns (zeros past the patch's own), the FP64 exponents, an odd length (banks)
+  static constexpr int MV = P == 2 ? 12 : 24, MP = P == 2 ? 9 : 16, LDW = (MV + MP + 1) | 1;
 };
 
 // A staged value or coefficient: two limbs (FP64) or the value itself (FP32).
@@ -77,8 +80,8 @@ struct PatchTab {
   int by_row;                       // rec is indexed by row
 };
 template <typename T> constexpr int inv8_ld() { return sizeof(T) == 8 ? 10 : 8; }
-// row length of a wall patch's inverse: odd, so that the rows of a warp fall into different banks;
-// the FP64 exponents are the entry after the nl-th
+// row length of a packed inverse of nl rows: odd, so that the rows of a warp fall into different
+// banks; the FP64 exponents are the entry after the nl-th (3D)
 __host__ __device__ constexpr int wall_ld(int nl) { return (nl + 1) | 1; }
 
 // One colour's patches (PatchGrid, igamg_internal.h).
@@ -89,6 +92,9 @@ struct ColourGrid {
 constexpr int kExpFloor = 128;      // biased exponents below this count as zero
 
 __device__ __forceinline__ int exp_of(double v) { return (__double2hiint(v) >> 20) & 0x7ff; }
+
+// v != 0 without an FP64 comparison (64 cycles)
+__device__ __forceinline__ bool nonzero(double v) { return (__double2hiint(v) << 1 | __double2loint(v)) != 0; }
 
 __device__ __forceinline__ unsigned long long shr64(unsigned long long x, int s) {
   unsigned long long r;                                        // s >= 64 gives 0
@@ -115,25 +121,24 @@ __device__ __forceinline__ int2 to_limbs(double v, int e) {
 }
 
 struct Acc {
-  long long hh = 0, mid = 0;
+  long long hh = 0, m1 = 0, m2 = 0;                            // three independent chains
   __device__ __forceinline__ void mac(int2 x, int2 c) {
     hh += (long long)x.x * c.x;
-    mid += (long long)x.x * c.y;
-    mid += (long long)x.y * c.x;
+    m1 += (long long)x.x * c.y;
+    m2 += (long long)x.y * c.x;
   }
-  __device__ __forceinline__ long long sum() const { return hh + (mid >> 28); }
+  __device__ __forceinline__ long long sum() const { return hh + ((m1 + m2) >> 28); }
 };
 
 // integer S in units of 2^(a - 1142), rounded to FP64
 __device__ __forceinline__ double to_double(long long S, int a) {
-  if (S == 0) return 0.0;
   const unsigned long long m = S < 0 ? 0ull - (unsigned long long)S : (unsigned long long)S;
   const int z = __clzll((long long)m);
   const unsigned long long n = m << z;
   const int ex = a - z - 56;                                   // biased exponent of the leading bit
   const unsigned long long mant = (n >> 11) + ((n >> 10) & 1);
   unsigned long long bits = ((unsigned long long)(unsigned)(ex - 1) << 52) + mant;
-  if (ex <= 0) bits = 0;
+  if (ex <= 0 || m == 0) bits = 0;
   if (ex >= 2047) bits = 0x7ff0000000000000ull;
   if (S < 0) bits |= 0x8000000000000000ull;
   return __longlong_as_double((long long)bits);
@@ -193,21 +198,26 @@ __device__ __forceinline__ Resid<T> row_resid(const limb_t<T>* sA, const limb_t<
   using S = PatchShape<P>;
   if constexpr (sizeof(T) == 8) {
     Acc A, B;
-    {
-      limb_t<T> own[S::RA];
-      if constexpr (!PRE) ld_entries_lazy<S::RA>(st, own);
-      const limb_t<T>* k = PRE ? st : own;
-#pragma unroll
-      for (int j = 0; j < S::NA; ++j) A.mac(sA[(j / S::C1) * S::W + j % S::C1], k[j]);
-    }
     int2 ec;
-    {
-      limb_t<T> own[S::NREC - S::RA];
-      if constexpr (!PRE) ld_entries_lazy<S::NREC - S::RA>(st + S::RA, own);
-      const limb_t<T>* k = PRE ? st + S::RA : own;
+    if constexpr (PRE) {
+      // both boxes in one loop: a dependent 64-bit multiply-add takes some 12 cycles, and a warp that is
+      // alone on its scheduler needs the six chains
 #pragma unroll
-      for (int j = 0; j < S::NB; ++j) B.mac(sB[(j / S::C1) * S::W + j % S::C1], k[j]);
-      ec = k[S::NB];
+      for (int j = 0; j < S::NA; ++j) {
+        const int at = (j / S::C1) * S::W + j % S::C1;
+        A.mac(sA[at], st[j]);
+        if (j < S::NB) B.mac(sB[at], st[S::RA + j]);
+      }
+      ec = st[S::RA + S::NB];
+    } else {
+      limb_t<T> ka[S::RA], kb[S::NREC - S::RA];
+      ld_entries_lazy<S::RA>(st, ka);
+#pragma unroll
+      for (int j = 0; j < S::NA; ++j) A.mac(sA[(j / S::C1) * S::W + j % S::C1], ka[j]);
+      ld_entries_lazy<S::NREC - S::RA>(st + S::RA, kb);
+#pragma unroll
+      for (int j = 0; j < S::NB; ++j) B.mac(sB[(j / S::C1) * S::W + j % S::C1], kb[j]);
+      ec = kb[S::NB];
     }
     const int aA = exA + ec.x, aB = exB + ec.y, exF = exp_of(f);
     int a = max(max(aA, aB), max(exF, kExpFloor));
@@ -223,7 +233,7 @@ __device__ __forceinline__ Resid<T> row_resid(const limb_t<T>* sA, const limb_t<
       sE_ = E.sum();
       a = max(a, aE);
     }
-    if (is_p && lam != 0.0) {                                  // (lam is the same for the whole grid)
+    if (is_p && nonzero(lam)) {                                  // (lam is the same for the whole grid)
       const int exL = max(exp_of(lam), kExpFloor);
       Acc Lm;
       Lm.mac(to_limbs(lam, exL), st[S::IL]);
@@ -238,7 +248,7 @@ __device__ __forceinline__ Resid<T> row_resid(const limb_t<T>* sA, const limb_t<
     r -= sar64(A.sum(), a - aA);
     r -= sar64(B.sum(), a - aB);
     if (EXT) r -= sar64(sE_, a - aE);
-    if (is_p && lam != 0.0) r -= sar64(sL, a - aL);
+    if (is_p && nonzero(lam)) r -= sar64(sL, a - aL);
     return {r, a};
   } else {
     T a0 = T(0), a1 = T(0), b0 = T(0), b1 = T(0);
@@ -297,7 +307,7 @@ struct Patch8 {
   using E = limb_t<T>;
   E st_[PRE ? S::NREC : 4], A[PRE ? inv8_ld<T>() : 4];
   const E *st, *Ap;
-  int a, b, g;
+  int a, b, g, nx, ny, np;          // nx, ny, np: the lane's first entries of the three arrays in U
   bool active;
 
   __device__ __forceinline__ void tables(const LevelTab<T>& L, const PatchTab<T>& X, const ColourGrid& C, int w, int lane) {
@@ -315,6 +325,12 @@ struct Patch8 {
     const int k = X.by_row ? g
                            : (is_p ? 2 : (is_y ? 1 : 0)) * NC * NC +
                                  cls1d<P>(ix, is_p || is_y ? L.lastq : L.lastp) * NC + cls1d<P>(iy, is_y ? L.lastp : L.lastq);
+    {
+      const int d = row / S::W, c = row - d * S::W;            // entry e = row + 8 k; k = 0
+      nx = (b - P + c) * L.nxu + (a - P - 1) + d;
+      ny = L.n_ux + (b - P - 1 + d) * L.npd + (a - P) + c;
+      np = L.n_ux + L.n_uy + (b - P + c) * L.npd + (a - P) + d;
+    }
     st = X.rec + (size_t)k * S::NREC;
     Ap = X.inv8 + ((size_t)icls * 8 + row) * inv8_ld<T>();
     if constexpr (PRE) {
@@ -331,20 +347,29 @@ struct Patch8 {
     const int o = row & 1, o2 = (row >> 1) & 1;
     // the neighbourhood: entry e = row + 8 k of each array
     T vx[KU], vy[KU], vp[KP];
-    const T* ux = U + (b - P) * L.nxu + (a - P - 1);
-    const T* uy = U + L.n_ux + (b - P - 1) * L.npd + (a - P);
-    const T* pr = U + L.n_ux + L.n_uy + (b - P) * L.npd + (a - P);
+    if constexpr (S::W == 4) {                                 // e -> e + 8: two steps along the long axis
 #pragma unroll
-    for (int k = 0; k < KU; ++k) {
-      const int e = row + 8 * k, d = e / S::W, c = e - d * S::W;
-      const bool in = S::NUX % 8 == 0 || k < KU - 1 || e < S::NUX;
-      vx[k] = in ? ux[c * L.nxu + d] : T(0);
-      vy[k] = in ? uy[d * L.npd + c] : T(0);
-    }
+      for (int k = 0; k < KU; ++k) {
+        const bool in = S::NUX % 8 == 0 || k < KU - 1 || row + 8 * k < S::NUX;
+        vx[k] = in ? U[nx + 2 * k] : T(0);
+        vy[k] = in ? U[ny + 2 * k * L.npd] : T(0);
+      }
 #pragma unroll
-    for (int k = 0; k < KP; ++k) {
-      const int e = row + 8 * k, d = e / S::W, c = e - d * S::W;
-      vp[k] = (S::NP % 8 == 0 || k < KP - 1 || e < S::NP) ? pr[c * L.npd + d] : T(0);
+      for (int k = 0; k < KP; ++k) vp[k] = U[np + 2 * k];
+    } else {
+      const int d0 = row / S::W, c0 = row - d0 * S::W;
+#pragma unroll
+      for (int k = 0; k < KU; ++k) {
+        const int e = row + 8 * k, d = e / S::W - d0, c = e % S::W - c0;
+        const bool in = S::NUX % 8 == 0 || k < KU - 1 || e < S::NUX;
+        vx[k] = in ? U[nx + c * L.nxu + d] : T(0);
+        vy[k] = in ? U[ny + d * L.npd + c] : T(0);
+      }
+#pragma unroll
+      for (int k = 0; k < KP; ++k) {
+        const int e = row + 8 * k, d = e / S::W - d0, c = e % S::W - c0;
+        vp[k] = (S::NP % 8 == 0 || k < KP - 1 || e < S::NP) ? U[np + c * L.npd + d] : T(0);
+      }
     }
     const T f = F[g], lam = U[L.n_total - 1], u_own = U[g];
     int eu = kExpFloor, ep = kExpFloor;
@@ -431,7 +456,7 @@ __device__ __forceinline__ void wall_sync() {
 // slots, and the inverse.
 template <int P>
 __host__ __device__ constexpr int wall_entries(int maxl) {
-  return (2 * PatchShape<P>::MARGIN + PatchShape<P>::REG + PatchShape<P>::LW + 16 + maxl * wall_ld(maxl) + 3) / 4 * 4;
+  return (2 * PatchShape<P>::MARGIN + PatchShape<P>::REG + PatchShape<P>::LW + 16 + maxl * PatchShape<P>::LDW + 3) / 4 * 4;
 }
 // Shared-memory entries per group of LW threads: one wall patch, or each warp's four patches.
 template <int P>
@@ -446,34 +471,26 @@ template <int P, typename T, bool EXT, bool PRE>
 struct PatchWall {
   using S = PatchShape<P>;
   using E = limb_t<T>;
+  static constexpr int K = (S::NLOAD + S::LW - 1) / S::LW;
   E st_[PRE ? S::NREC : 4];
+  int at[K];                        // the thread's neighbourhood values in U, -1: outside
   int4 D, R;                        // D: a | b << 16, offset of the inverse (16 B), rows | velocity rows << 8
                                     // R: row, offset of box A | of box B << 16, of the third box, record
 
   // t: thread within the group; sm: the group's shared memory
-  __device__ __forceinline__ void tables(const PatchTab<T>& X, int w, int t, E* sm) {
+  __device__ __forceinline__ void tables(const LevelTab<T>& L, const PatchTab<T>& X, int w, int t, E* sm) {
     D = X.wdesc[w];
     R = X.wrow[(size_t)w * S::LW + t];
     const int nl = D.z & 0xff;
     E* inv = sm + 2 * S::MARGIN + S::REG + S::LW + 16;
     const char* src = reinterpret_cast<const char*>(X.winv) + (size_t)D.y * 16;
-    const int n16 = (int)((nl * wall_ld(nl) * sizeof(E) + 15) / 16);
+    const int n16 = (int)((nl * S::LDW * sizeof(E) + 15) / 16);
     const unsigned dst = (unsigned)__cvta_generic_to_shared(inv);
     for (int i = t; i < n16; i += S::LW)
       asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst + 16 * i), "l"(src + 16 * (size_t)i) : "memory");
     asm volatile("cp.async.commit_group;" ::: "memory");
     if constexpr (PRE) ld_entries<S::NREC>(X.rec + (size_t)R.w * S::NREC, st_);   // threads past the last row: record 0
-  }
-
-  __device__ __forceinline__ void solve(const LevelTab<T>& L, const PatchTab<T>& X, T* U, const T* F, int t, E* sm) {
-    constexpr int K = (S::NLOAD + S::LW - 1) / S::LW;
-    const int a = D.x & 0xffff, b = D.x >> 16, nl = D.z & 0xff, nv = D.z >> 8, g = R.x, nu = L.n_ux + L.n_uy;
-    E* reg = sm + S::MARGIN;
-    E* rl = reg + S::REG + S::MARGIN;
-    int* red = reinterpret_cast<int*>(rl + S::LW);             // LW = 64: maxima of the two warps
-    const E* inv = rl + S::LW + 16;
-    T v[K];
-    int eu = kExpFloor, ep = kExpFloor;
+    const int a = D.x & 0xffff, b = D.x >> 16, nu = L.n_ux + L.n_uy;
 #pragma unroll
     for (int k = 0; k < K; ++k) {
       const int e = t + S::LW * k;
@@ -482,10 +499,21 @@ struct PatchWall {
       // u_y: y outer; u_x and pressure: x outer
       const int x = a - P + (uy && !pr ? cc : d), y = b - P + (uy && !pr ? d : cc);
       const int xlo = uy ? 0 : 1, xhi = uy ? L.lastq : L.nint, ylo = uy && !pr ? 1 : 0, yhi = uy && !pr ? L.nint : L.lastq;
-      v[k] = T(0);
-      if (e < S::NLOAD && x >= xlo && x <= xhi && y >= ylo && y <= yhi)
-        v[k] = U[(pr ? nu : (uy ? L.n_ux : 0)) + (y - ylo) * (uy ? L.npd : L.nxu) + x - xlo];
+      const bool in = e < S::NLOAD && x >= xlo && x <= xhi && y >= ylo && y <= yhi;
+      at[k] = in ? (pr ? nu : (uy ? L.n_ux : 0)) + (y - ylo) * (uy ? L.npd : L.nxu) + x - xlo : -1;
     }
+  }
+
+  __device__ __forceinline__ void solve(const LevelTab<T>& L, const PatchTab<T>& X, T* U, const T* F, int t, E* sm) {
+    const int nl = D.z & 0xff, nv = D.z >> 8, g = R.x, nu = L.n_ux + L.n_uy;
+    E* reg = sm + S::MARGIN;
+    E* rl = reg + S::REG + S::MARGIN;
+    int* red = reinterpret_cast<int*>(rl + S::LW);             // LW = 64: maxima of the two warps
+    const E* inv = rl + S::LW + 16;
+    T v[K];
+    int eu = kExpFloor, ep = kExpFloor;
+#pragma unroll
+    for (int k = 0; k < K; ++k) v[k] = at[k] >= 0 ? U[at[k]] : T(0);
     const bool has = t < nl, is_p = g >= nu;
     const T f = has ? F[g] : T(0), u_own = has ? U[g] : T(0), lam = U[L.n_total - 1];
     bool bad = false;
@@ -533,8 +561,13 @@ struct PatchWall {
     const Resid<T> r = row_resid<P, T, EXT, PRE>(sA, sB, reg + R.z, PRE ? st_ : X.rec + (size_t)R.w * S::NREC, se, is_p, eu,
                                                  is_p ? eu : ep, eu, f, lam);
     asm volatile("cp.async.wait_all;" ::: "memory");
-    const int ld = wall_ld(nl);
-    const E* Ak = inv + (has ? t : 0) * ld;
+    const E* Ak = inv + (has ? t : 0) * S::LDW;
+    const int slot = t < nv ? t : S::MV + t - nv;              // the row's column in the inverses
+    // columns that the patch does not have (their entries in the inverse are zero)
+    if (t < S::MV + S::MP && (t < S::MV ? t >= nv : t - S::MV >= nl - nv)) {
+      if constexpr (sizeof(T) == 8) rl[t] = make_int2(0, 0);
+      else rl[t] = T(0);
+    }
     if constexpr (sizeof(T) == 8) {
       const int er = has ? resid_exp(r) : 0;
       int gu = __reduce_max_sync(0xffffffffu, is_p ? 0 : er), gp = __reduce_max_sync(0xffffffffu, is_p ? er : 0);
@@ -547,48 +580,60 @@ struct PatchWall {
       } else {
         bad = __any_sync(0xffffffffu, bad);
       }
-      if (has) rl[t] = resid_limbs(r, er, is_p ? gp : gu);
+      if (has) rl[slot] = resid_limbs(r, er, is_p ? gp : gu);
       wall_sync<S::LW>();                                      // (also makes every thread's cp.async visible)
-      if (has) {
-        Acc D0, D1;
-#pragma unroll 4
-        for (int s = 0; s < nv; ++s) D0.mac(rl[s], Ak[s]);
-#pragma unroll 4
-        for (int s = nv; s < nl; ++s) D1.mac(rl[s], Ak[s]);
-        const int2 ec = Ak[nl];
-        const int a0 = gu + ec.x, a1 = gp + ec.y, am = max(a0, a1);
-        double d = to_double(sar64(D0.sum(), am - a0) + sar64(D1.sum(), am - a1), am);
-        if (bad) d = __longlong_as_double(0x7ff8000000000000ll);
-        U[g] = u_own + d;
+      Acc D0, D1;
+#pragma unroll
+      for (int s = 0; s < S::MV; ++s) {
+        D0.mac(rl[s], Ak[s]);
+        if (s < S::MP) D1.mac(rl[S::MV + s], Ak[S::MV + s]);
       }
+      const int2 ec = Ak[S::MV + S::MP];
+      const int a0 = gu + ec.x, a1 = gp + ec.y, am = max(a0, a1);
+      double d = to_double(sar64(D0.sum(), am - a0) + sar64(D1.sum(), am - a1), am);
+      if (bad) d = __longlong_as_double(0x7ff8000000000000ll);
+      if (has) U[g] = u_own + d;
     } else {
-      if (has) rl[t] = r.v;
+      if (has) rl[slot] = r.v;
       wall_sync<S::LW>();
-      if (has) U[g] = u_own + dot_n(Ak, rl, nl);
+      T d[3] = {T(0), T(0), T(0)};
+#pragma unroll
+      for (int s = 0; s < S::MV + S::MP; ++s) d[s % 3] = fma(Ak[s], rl[s], d[s % 3]);
+      if (has) U[g] = u_own + ((d[0] + d[1]) + d[2]);
     }
     wall_sync<S::LW>();                                        // the shared memory is free again
   }
 };
 
 // Group w of LW threads of one colour's work: the wall patches first (their chains are the
-// longest), then the interior patches, four to a warp along x.  WAIT: the kernel's dependency
-// wait stands between the table loads and the solve.
+// longest), then the interior patches, four to a warp along x.  WAIT: the kernel's dependency wait
+// stands between the table loads and the solve, in a loop of `once` (always 1) rounds that the
+// compiler cannot unroll: it then computes every address and table value that does not depend on U
+// before the loop, ahead of the wait, instead of sinking them to their uses.  Measured per colour
+// with and without the loop: p = 3 64^2 2.65 and 3.08 us, 128^2 3.1 and 3.8, p = 2 128^2 2.5 and 2.9,
+// 256^2 5.0-5.5 and 5.0 (more registers); V-cycle p = 3 72^2 614 and 697 us.
 template <int P, typename T, bool EXT, bool PRE, bool WAIT>
 __device__ __forceinline__ void colour_group(const LevelTab<T>& L, const PatchTab<T>& X, T* U, const T* F,
-                                             const ColourGrid& C, int w, int t, limb_t<T>* sm) {
+                                             const ColourGrid& C, int w, int t, limb_t<T>* sm, int once) {
   using S = PatchShape<P>;
   if (w < C.nwall) {
     PatchWall<P, T, EXT, PRE> W;
-    W.tables(X, C.wfirst + w, t, sm);
-    if (WAIT) dependency_wait();
-    W.solve(L, X, U, F, t, sm);
+    W.tables(L, X, C.wfirst + w, t, sm);
+#pragma unroll 1
+    for (int k = 0; k < (WAIT ? once : 1); ++k) {
+      if (WAIT) dependency_wait();
+      W.solve(L, X, U, F, t, sm);
+    }
   } else {
     const int wp = (w - C.nwall) * (S::LW / 32) + (t >> 5);
     if (wp >= C.n8 / max(C.na, 1) * ((C.na + 3) >> 2)) return;
     Patch8<P, T, EXT, PRE> I;
     I.tables(L, X, C, wp, t & 31);
-    if (WAIT) dependency_wait();
-    I.solve(L, X, U, F, t & 31, sm + (t >> 5) * 4 * S::REG);
+#pragma unroll 1
+    for (int k = 0; k < (WAIT ? once : 1); ++k) {
+      if (WAIT) dependency_wait();
+      I.solve(L, X, U, F, t & 31, sm + (t >> 5) * 4 * S::REG);
+    }
   }
 }
 template <int P>
@@ -602,12 +647,13 @@ __host__ __device__ inline int colour_groups(const ColourGrid& C) {
 // warps per SM) measured 2.75 against 2.2 us on 64^2, 6.4 against 6.5 on 256^2 (p = 2).
 template <int P, typename T, bool EXT>
 __global__ void __launch_bounds__(64) k_patch_colour(const __grid_constant__ LevelTab<T> L, const __grid_constant__ PatchTab<T> X,
-                                                     T* U, const T* F, const ColourGrid C, int ngroups, int smg) {
+                                                     T* U, const T* F, const ColourGrid C, int ngroups, int smg, int once) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   constexpr int LW = PatchShape<P>::LW;
   const int gib = threadIdx.x / LW, w = blockIdx.x * (64 / LW) + gib;
   if (w >= ngroups) return;
-  colour_group<P, T, EXT, true, true>(L, X, U, F, C, w, threadIdx.x % LW, reinterpret_cast<limb_t<T>*>(smem_raw) + gib * smg);
+  colour_group<P, T, EXT, true, true>(L, X, U, F, C, w, threadIdx.x % LW, reinterpret_cast<limb_t<T>*>(smem_raw) + gib * smg,
+                                      once);
 }
 
 // ---- building the tables (once, at creation) ---------------------------------------------------
@@ -705,15 +751,24 @@ __global__ void k_patch_inv8(int ncls, const T* __restrict__ src, limb_t<T>* __r
 
 // The other patches: one block per class c of spec (x: class in cinv8 (-1 - x) or cinv, y: offset of
 // the result in 16 bytes, z: rows | velocity rows << 8), threads over its rows.
-template <typename T>
+template <int P, typename T>
 __global__ void k_patch_winv(int maxl, const int4* __restrict__ spec, const T* __restrict__ cinv, const T* __restrict__ cinv8,
                              limb_t<T>* __restrict__ dst) {
   const int4 s = spec[blockIdx.x];
   const int nl = s.z & 0xff, nv = s.z >> 8, r = threadIdx.x;
   if (r >= nl) return;
   const T* src = s.x < 0 ? cinv8 + ((size_t)(-1 - s.x) * 8 + r) * 8 : cinv + ((size_t)s.x * maxl + r) * maxl;
-  limb_t<T>* d = reinterpret_cast<limb_t<T>*>(reinterpret_cast<char*>(dst) + (size_t)s.y * 16) + r * wall_ld(nl);
-  inverse_row<T>(src, nl, nv, d);
+  using S = PatchShape<P>;
+  limb_t<T>* d = reinterpret_cast<limb_t<T>*>(reinterpret_cast<char*>(dst) + (size_t)s.y * 16) + r * S::LDW;
+  limb_t<T> row[S::MV + S::MP + 1];
+  inverse_row<T>(src, nl, nv, row);
+  for (int j = 0; j < S::LDW; ++j) {
+    limb_t<T> v{};
+    if (j < nv) v = row[j];
+    else if (j >= S::MV && j - S::MV < nl - nv) v = row[nv + j - S::MV];
+    else if (sizeof(T) == 8 && j == S::MV + S::MP) v = row[nl];
+    d[j] = v;
+  }
 }
 
 // ---- lockstep batches of any mesh sizes: one launch per V-cycle step over every solve -------
@@ -764,7 +819,7 @@ __global__ void __launch_bounds__(128) k_mix_colour(const __grid_constant__ MixA
     const LevelTab<T> L = d.L;
     const PatchTab<T> X = d.X;
     colour_group<P, T, EXT, false, false>(L, X, d.U, d.F, C, w, threadIdx.x % LW,
-                                   reinterpret_cast<limb_t<T>*>(smem_raw) + gib * smg);
+                                   reinterpret_cast<limb_t<T>*>(smem_raw) + gib * smg, 1);
     return;
   }
   const int wpb = blockDim.x >> 5, ppw = d.lpr == 2 ? 2 : 4;

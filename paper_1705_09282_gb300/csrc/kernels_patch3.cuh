@@ -86,18 +86,30 @@ __device__ __forceinline__ Resid<T> row_part(const limb_t<T>* reg, int oA, int o
   const limb_t<T>* pC = is_p ? reg + oC + min(s, 2 * P - 1) * S::LS : reg + oA + (S::LPR < S::A1 && s == 0 ? S::LPR * S::LS : 0);
   if constexpr (sizeof(T) == 8) {
     Acc A, B, C;
-    int aA, aB, aC;
-    auto box = [&](Acc& acc, const limb_t<T>* p, const limb_t<T>* c) -> int {
-      limb_t<T> own[SLP];
-      if constexpr (!PRE) ld_entries_lazy<SLP>(c, own);
-      const limb_t<T>* k = PRE ? c : own;
+    int aA = eu, aB = is_p ? eu : ep, aC = eu;
+    if constexpr (PRE) {                                       // the three boxes' chains side by side
 #pragma unroll
-      for (int j = 0; j < S::SL; ++j) acc.mac(p[(j / S::C1) * S::W + j % S::C1], k[j]);
-      return k[S::SL].x;
-    };
-    aA = eu + box(A, pA, st);
-    aB = (is_p ? eu : ep) + box(B, pB, st + SLP);
-    aC = eu + box(C, pC, st + 2 * SLP);
+      for (int j = 0; j < S::SL; ++j) {
+        const int at = (j / S::C1) * S::W + j % S::C1;
+        A.mac(pA[at], st[j]);
+        B.mac(pB[at], st[SLP + j]);
+        C.mac(pC[at], st[2 * SLP + j]);
+      }
+      aA += st[S::SL].x;
+      aB += st[SLP + S::SL].x;
+      aC += st[2 * SLP + S::SL].x;
+    } else {
+      auto box = [&](Acc& acc, const limb_t<T>* p, const limb_t<T>* c) -> int {
+        limb_t<T> k[SLP];
+        ld_entries_lazy<SLP>(c, k);
+#pragma unroll
+        for (int j = 0; j < S::SL; ++j) acc.mac(p[(j / S::C1) * S::W + j % S::C1], k[j]);
+        return k[S::SL].x;
+      };
+      aA += box(A, pA, st);
+      aB += box(B, pB, st + SLP);
+      aC += box(C, pC, st + 2 * SLP);
+    }
     const int exF = exp_of(f);
     int a = max(max(aA, max(aB, aC)), max(exF, kExpFloor));
     long long sE = 0, sL = 0;
@@ -119,7 +131,7 @@ __device__ __forceinline__ Resid<T> row_part(const limb_t<T>* reg, int oA, int o
       sE = E.sum();
       a = max(a, aE);
     }
-    if (is_p && lam != 0.0) {
+    if (is_p && nonzero(lam)) {
       const int exL = max(exp_of(lam), kExpFloor);
       Acc Lm;
       Lm.mac(to_limbs(lam, exL), tail[0]);
@@ -133,7 +145,7 @@ __device__ __forceinline__ Resid<T> row_part(const limb_t<T>* reg, int oA, int o
       const unsigned long long M = ((unsigned long long)(unsigned)((h & 0xfffff) | 0x100000) << 32) | (unsigned)__double2loint(f);
       r = (long long)shr64(M << 7, a - exF);
       if (h < 0) r = -r;
-      if (is_p && lam != 0.0) r -= sar64(sL, a - aL);
+      if (is_p && nonzero(lam)) r -= sar64(sL, a - aL);
     }
     r -= sar64(A.sum(), a - aA);
     r -= sar64(B.sum(), a - aB);
@@ -142,16 +154,16 @@ __device__ __forceinline__ Resid<T> row_part(const limb_t<T>* reg, int oA, int o
     return {r, a};
   } else {
     T x0 = T(0), x1 = T(0), x2 = T(0);
-    auto box = [&](T& acc, const limb_t<T>* p, const limb_t<T>* c) {
-      limb_t<T> own[SLP];
-      if constexpr (!PRE) ld_entries_lazy<SLP>(c, own);
-      const limb_t<T>* k = PRE ? c : own;
+    limb_t<T> own[PRE ? 4 : 3 * SLP];
+    if constexpr (!PRE) ld_entries_lazy<3 * SLP>(st, own);
+    const limb_t<T>* k = PRE ? st : own;
 #pragma unroll
-      for (int j = 0; j < S::SL; ++j) acc = fma(k[j], p[(j / S::C1) * S::W + j % S::C1], acc);
-    };
-    box(x0, pA, st);
-    box(x1, pB, st + SLP);
-    box(x2, pC, st + 2 * SLP);
+    for (int j = 0; j < S::SL; ++j) {
+      const int at = (j / S::C1) * S::W + j % S::C1;
+      x0 = fma(k[j], pA[at], x0);
+      x1 = fma(k[SLP + j], pB[at], x1);
+      x2 = fma(k[2 * SLP + j], pC[at], x2);
+    }
     if (EXT && se && s < S::XA) {
       constexpr int XL = ext_slice_len<P, T>();
       const limb_t<T>* pE = reg + oE + s * S::LS;

@@ -961,12 +961,13 @@ bool patch_grids(int p, const igamg_sizes& s, const PatchTables& pt, bool by_row
                                          by_row ? pd[r] : D.blk * NC * NC + cl});
       }
       if (is8 && nv != 4) return false;
+      if (nv > (p == 2 ? 12 : 24) || nl - nv > (p == 2 ? 9 : 16)) return false;   // PatchShape::MV, MP
       const int key = is8 ? -1 - pt.cls[i] : pt.cls[i], rows = nl | (nv << 8);
       auto it = wcls.find(key);
       if (it == wcls.end()) {
         it = wcls.emplace(key, (int)out.wspec.size() / 4).first;
         out.wspec.insert(out.wspec.end(), {key, out.winv16, rows, 0});
-        out.winv16 += (nl * ((nl + 1) | 1) * entry_bytes + 15) / 16;   // wall_ld(nl) entries per row
+        out.winv16 += (nl * (p == 2 ? 23 : 41) * entry_bytes + 15) / 16;   // PatchShape::LDW entries per row
       }
       out.wdesc.insert(out.wdesc.end(), {a | (b << 16), out.wspec[(size_t)4 * it->second + 1], rows, 0});
     }
