@@ -300,7 +300,7 @@ def run_ours(args):
 
     # ---- dominant kernel: the finest level's multiplicative sweep ------------------------
     # nu = 2 sweeps (all colours) of the finest level, as in every V-cycle's pre- and
-    # post-smoothing, in the form the autotuner chose for that level, captured into a CUDA
+    # post-smoothing, in the form that level runs, captured into a CUDA
     # graph (the way solves run it) on a side stream and replayed 10 times between CUDA
     # events on that stream; the average per colour launch (or per pipelined launch) is the
     # kernel's launch duration.
@@ -358,7 +358,12 @@ def run_ours(args):
     # algorithmic bytes per sweep: U read and written once, F read once, the patch DOF lists
     # (8 int32 per patch) and class ids read once
     bytes_replay = sweeps_per_replay * (3 * 8 * sz.n_total + sz.n_patches * (8 + 1) * 4)
-    if form["tiles"]:
+    pins = ("IGAMG_SWEEP_FORM", "IGAMG_ROW_LANES", "IGAMG_TILE_MULT", "IGAMG_SPLIT_COLOUR")
+    staged = not any(k in os.environ for k in pins)     # the row kernels run only where a variable pins them
+    if staged:
+        kname = (f"k_patch_colour<{p0},double> (one colour of the finest level {N_FINE}^2, staged "
+                 "neighbourhoods, 64-thread blocks)")
+    elif form["tiles"]:
         kname = (f"k_sweep_tiles<{p0},double> (pipelined: {form['tiles']} tiles of {form['threads']} threads; "
                  f"one launch = 2 sweeps x {sz.n_colours} colours)")
     else:
@@ -369,7 +374,7 @@ def run_ours(args):
     # (colours 0 and 1 of the 256^2 finest level, mean of the two launches), for the forms
     # captured; none for another form
     captured = {(1, 64, 0, 4): 3.21e6, (1, 64, 0, 2): 3.208e6}
-    traffic = captured.get((form["lanes"], form["threads"], form["tiles"], form["chains"])) if p0 == 2 else None
+    traffic = captured.get((form["lanes"], form["threads"], form["tiles"], form["chains"])) if p0 == 2 and not staged else None
     roofline = {"kernel": kname, "bound": "alu",
                 "achieved": achieved, "peak": fp64_peak, "unit": "TFLOP/s (FP64)", "frac": achieved / fp64_peak,
                 "traffic": traffic, "traffic_unit": "bytes per launch",
@@ -384,7 +389,8 @@ def run_ours(args):
                 "achieved_gbs_algorithmic": bytes_replay / t_sweeps / 1e9,
                 "hbm_peak_gbs": pk["hbm_gbs"], "hbm_peak_source": pk_src, "form": form,
                 "timing": "2 sweeps captured in a CUDA graph on a side stream, 10 replays between CUDA events",
-                "working_set_note": "finest-level vectors (1.6 MB) stay in L2; the kernel is FP64-issue bound"}
+                "working_set_note": "finest-level vectors (1.6 MB) stay in L2; a colour is bound by the "
+                                    "dependent chain of one patch solve"}
     # the FP32 inner smoother of the mixed mode, same launches
     bytes32 = sweeps_per_replay * (3 * 4 * sz.n_total + sz.n_patches * (8 + 1) * 4)
     roofline32 = {"kernel": kname.replace(",double", ",float").replace(f",{form['chains']}>", ",4>").replace(

@@ -171,7 +171,8 @@ int igamg_residual(igamg_handle* h, int level, const double* U, const double* F,
 /* `sweeps` applications of the level's Schwarz smoother to U in place (Sec. 5.2). */
 int igamg_smooth(igamg_handle* h, int level, double* U, const double* F, int sweeps);
 
-/* The form of level `level`'s multiplicative sweep that the autotuner chose at creation (2D):
+/* The form of level `level`'s multiplicative sweep, chosen at creation (2D; a level that runs the
+ * staged colour kernels reports one lane, 64 threads and no tiles):
  * *lanes = lanes per local row of the 8-DOF patches (1 or 2), *threads = threads per block,
  * *tiles = 0 for one launch per colour, else the number of tiles of the pipelined sweep
  * (1: the whole level in one block).  Any output may be NULL.  Errors: IGAMG_EINVAL,
