@@ -908,6 +908,14 @@ int batch_launches(igamg_handle** all, const std::vector<int>& idx, const std::v
     for (int i = 0; i < n; ++i) A[t].s[i] = mix[(size_t)idx[i] * nd + t];
   }
   const int tpb = 128, wpb = tpb / 32;
+  // of the whole group: a one-grid handle has no colours, and a level without staged tables (p = 3 on
+  // 4 x 4 elements) has a third box all the same
+  int C = 0;
+  bool ext = false;
+  for (int i = 0; i < n; ++i) {
+    C = std::max(C, hs[i]->lc.back().n_colours);
+    ext = ext || hs[i]->d.lev.back().L.sext != nullptr;
+  }
   auto lev = [&](int i, int t) { return (int)hs[i]->d.lev.size() - 1 - t; };
   auto max_over = [&](int t, int min_level, auto f) {
     long long m = 0;
@@ -921,7 +929,6 @@ int batch_launches(igamg_handle** all, const std::vector<int>& idx, const std::v
     k_mix_residual_finish<double><<<ns, 1024, 0, s>>>(A[t], any, want, kBlock);
   };
   auto smooth = [&](int t) {
-    const int C = hs[0]->lc.back().n_colours;
     // shared memory per group of a staged level, and per block of any level
     auto entries = [&](int i, int l) {
       const int m = hs[i]->lc[l].maxl;
@@ -931,7 +938,6 @@ int batch_launches(igamg_handle** all, const std::vector<int>& idx, const std::v
     const size_t shm = sizeof(double) * std::max((size_t)gpb * smg, (size_t)wpb * max_over(t, 1, [&](int i, int l) {
       return hs[i]->lc[l].staged ? 0 : hs[i]->lc[l].maxl;
     }));
-    const bool ext = hs[0]->d.lev.back().X.ext != nullptr;
     for (int c = 0; c < C; ++c) {
       unsigned nb = max_over(t, 1, [&](int i, int l) {
         const auto& lc = hs[i]->lc[l];

@@ -129,3 +129,36 @@ def test_member_handle_recreated_between_batches(monkeypatch):
     assert reps[1]["cycles"] == r1["cycles"]
     a, b = UC.cpu().numpy(), U1.cpu().numpy()
     assert np.abs(a - b).max() <= 1e-12 * np.abs(b).max()
+
+
+@pytest.mark.parametrize("cases", [
+    # p = 3 on 4 x 4 elements keeps the row kernels; the staged levels of the larger meshes behind it
+    # need their third box
+    [(3, 4, 2, 1.0, {"geometry": 1}), (3, 8, 2, 1e2, {"geometry": 1}), (3, 16, 3, 1e-2, {"geometry": 1})],
+    # a one-grid handle has no colours; the levels of the others have
+    [(2, 8, 1, 1.0, {}), (2, 16, 3, 1e2, {}), (2, 32, 4, 1e-2, {})],
+    [(3, 8, 1, 1.0, {}), (3, 16, 3, 1e2, {}), (3, 8, 2, 1e-2, {})],
+])
+def test_group_led_by_its_smallest_mesh(cases, monkeypatch):
+    # as _run, without the histories: a direct solve's residual is rounding
+    torch = _torch()
+    from paper_1705_09282_gb300.solver import Solver, solve_batch
+    monkeypatch.setenv("IGAMG_FUSED_LEVELS", "-1")
+    monkeypatch.setenv("IGAMG_LOCKSTEP_MIN", "2")
+    solvers = [Solver(p, n, L, sigma, 1.0, **kw) for p, n, L, sigma, kw in cases]
+    Fs, Us, singles = [], [], []
+    for j, (S, (p, n, L, sigma, kw)) in enumerate(zip(solvers, cases)):
+        if kw.get("geometry", 0) == 1:
+            X = S.quad_points_xy()
+            f = inputs.annulus_forcing(X[0], X[1], sigma, 1.0)
+        else:
+            f = inputs.grf_forcing(p, n, seed=900 + j)
+        F = S.load_vector(torch.tensor(f, device="cuda"))
+        U1 = S.empty()
+        singles.append((S.solve(U1, F, rtol=1e-8, max_cycles=80), U1))
+        Fs.append(F)
+        Us.append(S.empty())
+    reps = solve_batch(solvers, Us, Fs, rtol=1e-8, max_cycles=80)
+    for j, ((r1, U1), rep, U) in enumerate(zip(singles, reps, Us)):
+        assert rep["converged"] and r1["converged"] and rep["cycles"] == r1["cycles"], j
+        assert float((U - U1).abs().max()) <= 1e-12 * float(U1.abs().max()), j
