@@ -370,6 +370,11 @@ int igamg_residual_static(const igamg_problem* prob, int level, const double* U,
  * measured FMA throughput, the denominator of the roofline of FMA-issue-bound kernels.
  * Errors: IGAMG_EINVAL (non-positive sizes, null out), IGAMG_ECUDA (launch failed). */
 int igamg_probe_fma(int fp64, int blocks, int iters, void* out, void* cuda_stream, double* flops);
+/* Precision probe, not part of the method: the local residuals F - K U of every patch row of a
+ * level as the staged colour kernels form them (before the local inverses mix the rows), into
+ * R[0 .. n_total-2] (device; U and F are only read).  Enqueued on the handle's stream.  Errors:
+ * IGAMG_EINVAL, IGAMG_EUNSUPPORTED (the level does not run those kernels), IGAMG_ECUDA. */
+int igamg_probe_patch_rows(igamg_handle* h, int level, const double* U, const double* F, double* R);
 
 /* ---- host-only inspection of the set-up (no GPU needed; for tests) -------------------
  * Each call builds the hierarchy on the host and copies one piece out, dense, row-major.

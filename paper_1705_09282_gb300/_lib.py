@@ -79,6 +79,7 @@ SIGNATURES = {
     "igamg_curl": (_I, [_P, _P, _P]),
     "igamg_residual_static": (_I, [ctypes.POINTER(Problem), _I, _P, _P, _P, ctypes.POINTER(_D), _P]),
     "igamg_probe_fma": (_I, [_I, _I, _I, _P, _P, ctypes.POINTER(_D)]),
+    "igamg_probe_patch_rows": (_I, [_P, _I, _P, _P, _P]),
     "igamg_smooth_f32": (_I, [_P, _I, _P, _P, _I]),
     "igamg_residual_f32": (_I, [_P, _I, _P, _P, _P, _P]),
     "igamg_residual_form": (_I, [_P, ctypes.POINTER(_I), ctypes.POINTER(_I)]),

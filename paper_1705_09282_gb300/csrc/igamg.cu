@@ -445,6 +445,23 @@ int do_smooth_staged(igamg_handle* h, int l, T* U, const T* F, cudaStream_t s) {
   return IGAMG_OK;
 }
 
+// igamg_probe_patch_rows: the rows of every colour, no solves.
+template <int P>
+int do_patch_rows(igamg_handle* h, int l, const double* U, const double* F, double* R, cudaStream_t s) {
+  auto& lc = h->lc[l];
+  auto& tl = h->d.lev[l];
+  const int gpb = kPatchThreads / PatchShape<P>::LW, smg = group_entries<P>(lc.maxl);
+  const size_t shm = (size_t)gpb * smg * sizeof(limb_t<double>);
+  for (const ColourGrid& C : lc.grids) {
+    const int ng = colour_groups<P>(C);
+    if (ng == 0) continue;
+    const unsigned nb = (unsigned)((ng + gpb - 1) / gpb);
+    if (tl.X.ext) k_patch_rows<P, true><<<nb, kPatchThreads, shm, s>>>(tl.L, tl.X, const_cast<double*>(U), F, R, C, ng, smg);
+    else k_patch_rows<P, false><<<nb, kPatchThreads, shm, s>>>(tl.L, tl.X, const_cast<double*>(U), F, R, C, ng, smg);
+  }
+  return launch_check();
+}
+
 template <typename T>
 int do_smooth(igamg_handle* h, int l, T* U, const T* F, cudaStream_t s) {
   auto& lc = h->lc[l];
@@ -2388,6 +2405,14 @@ int igamg_smooth(igamg_handle* h, int level, double* U, const double* F, int swe
   if (h && U && F && h->d3) return h3_smooth(h->d3, level, U, F, sweeps);
   if (!h || !U || !F || level < 1 || level >= (int)h->lc.size() || sweeps < 0) return IGAMG_EINVAL;
   return do_smooth_n<double>(h, level, U, F, sweeps, h->stream);
+}
+
+int igamg_probe_patch_rows(igamg_handle* h, int level, const double* U, const double* F, double* R) {
+  if (!h || !U || !F || !R) return IGAMG_EINVAL;
+  if (h->d3) return h3_probe_patch_rows(h->d3, level, U, F, R);
+  if (level < 1 || level >= (int)h->lc.size()) return IGAMG_EINVAL;
+  if (!h->lc[level].staged) return IGAMG_EUNSUPPORTED;
+  return h->prob.p == 2 ? do_patch_rows<2>(h, level, U, F, R, h->stream) : do_patch_rows<3>(h, level, U, F, R, h->stream);
 }
 
 int igamg_level_form(const igamg_handle* h, int level, int* lanes, int* threads, int* tiles) {

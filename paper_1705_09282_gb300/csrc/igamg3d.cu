@@ -472,14 +472,30 @@ int do_smooth_staged(igamg3d_handle* h, int l, T* U, const T* F, cudaStream_t s)
     if (nb == 0) continue;
     cfg.gridDim = dim3((unsigned)nb);
     const bool pre = nb <= kPreBlocks;
+    T* const none = nullptr;
     cudaError_t e;
-    if (tl.X.ext) e = pre ? cudaLaunchKernelEx(&cfg, k_patch_colour3<P, T, true, true>, tl.L, tl.X, U, F, C)
-                          : cudaLaunchKernelEx(&cfg, k_patch_colour3<P, T, true, false>, tl.L, tl.X, U, F, C);
-    else e = pre ? cudaLaunchKernelEx(&cfg, k_patch_colour3<P, T, false, true>, tl.L, tl.X, U, F, C)
-                 : cudaLaunchKernelEx(&cfg, k_patch_colour3<P, T, false, false>, tl.L, tl.X, U, F, C);
+    if (tl.X.ext) e = pre ? cudaLaunchKernelEx(&cfg, k_patch_colour3<P, T, true, true>, tl.L, tl.X, U, F, C, none)
+                          : cudaLaunchKernelEx(&cfg, k_patch_colour3<P, T, true, false>, tl.L, tl.X, U, F, C, none);
+    else e = pre ? cudaLaunchKernelEx(&cfg, k_patch_colour3<P, T, false, true>, tl.L, tl.X, U, F, C, none)
+                 : cudaLaunchKernelEx(&cfg, k_patch_colour3<P, T, false, false>, tl.L, tl.X, U, F, C, none);
     if (e != cudaSuccess) { set_error(cudaGetErrorString(e)); return IGAMG_ECUDA; }
   }
   return IGAMG_OK;
+}
+
+// h3_probe_patch_rows: the rows of every colour, no solves.
+template <int P>
+int do_patch_rows(igamg3d_handle* h, int l, const double* U, const double* F, double* R, cudaStream_t s) {
+  using S = PatchShape3<P>;
+  auto& tl = h->d.lev[l];
+  const size_t shm = patch3_smem<P, double>(tl.X.maxl);
+  for (const ColourGrid3& C : h->lc[l].grids) {
+    const unsigned nb = (unsigned)(C.nwall + (C.n8 + S::PPB - 1) / S::PPB);
+    if (nb == 0) continue;
+    if (tl.X.ext) k_patch_colour3<P, double, true, true, true><<<nb, S::NT, shm, s>>>(tl.L, tl.X, const_cast<double*>(U), F, C, R);
+    else k_patch_colour3<P, double, false, true, true><<<nb, S::NT, shm, s>>>(tl.L, tl.X, const_cast<double*>(U), F, C, R);
+  }
+  return launch_check();
 }
 
 template <typename T>
@@ -987,6 +1003,12 @@ int h3_smooth(igamg3d_handle* h, int level, double* U, const double* F, int swee
   if (level < 1 || level >= (int)h->lc.size() || sweeps < 0) return IGAMG_EINVAL;
   for (int k = 0; k < sweeps; ++k) { int rc = do_smooth<double>(h, level, U, F, h->stream); if (rc) return rc; }
   return IGAMG_OK;
+}
+
+int h3_probe_patch_rows(igamg3d_handle* h, int level, const double* U, const double* F, double* R) {
+  if (level < 1 || level >= (int)h->lc.size()) return IGAMG_EINVAL;
+  if (!h->lc[level].staged) return IGAMG_EUNSUPPORTED;
+  return h->prob.p == 2 ? do_patch_rows<2>(h, level, U, F, R, h->stream) : do_patch_rows<3>(h, level, U, F, R, h->stream);
 }
 
 int h3_restrict(igamg3d_handle* h, int level, const double* r, double* g) {

@@ -21,6 +21,7 @@ const std::vector<double>& h3_quad_xyz(const igamg3d_handle* h);   // mapped dom
 int h3_load_vector(igamg3d_handle* h, const double* f_qp, double* F);
 int h3_residual(igamg3d_handle* h, int level, const double* U, const double* F, double* R, double* norm_out);
 int h3_smooth(igamg3d_handle* h, int level, double* U, const double* F, int sweeps);
+int h3_probe_patch_rows(igamg3d_handle* h, int level, const double* U, const double* F, double* R);
 int h3_restrict(igamg3d_handle* h, int level, const double* r, double* g);
 int h3_prolong_add(igamg3d_handle* h, int level, const double* uc, double* uf);
 int h3_coarse_solve(igamg3d_handle* h, const double* G, double* U);

@@ -7,16 +7,27 @@
 // to 4 warps per scheduler), a 32 x 32 + 64 bit integer multiply-add 2.3-2.6 cycles.  A patch row
 // of degree p = 2 (27 stencil terms, 8 columns of the local inverse) costs some 45 FP64
 // instructions, 2900 cycles per warp.  Here every value of a patch's neighbourhood is turned once
-// into two integer limbs relative to the neighbourhood's largest exponent, and every product of
-// a coefficient with a value is three integer multiply-adds, exact up to its last bits:
+// into two integer limbs relative to the largest exponent of its component (u_x, u_y, u_z,
+// pressure) there, and every product of a coefficient with a value is three integer multiply-adds:
 //   value        v = (hi 2^28 + lo) 2^(e - 57),  |v| < 2^e, |hi| < 2^29, 0 <= |lo| < 2^28
 //   coefficient  c = (hi 2^28 + lo) 2^(s - 59),  sum of the box |c| < 2^(s-1),  |lo| <= 2^27
 //   sum_j c_j v_j = (HH + MID 2^-28) 2^(e + s - 60),  HH = sum hi hi, MID = sum (hi lo + lo hi)
-// The sums are exact in 64-bit integers (|HH| <= 2^59, |MID| < 2^62); what is dropped or
-// truncated is below 2^-57 of (largest value) x (sum of |coefficients|), against 2^-53 of the
-// running sum per FP64 rounding, so a row's error is smaller than the FP64 kernels'.  The local
-// residuals stay integers and go through the local inverse the same way (one exponent for the
-// velocity rows, one for the pressure rows); the correction is rounded once to FP64.
+// The sums are exact in 64-bit integers (|HH| <= 2^59, |MID| < 2^62).  A row's error is bounded per
+// box, relative to M = (the component's largest value in the neighbourhood) x (sum of the box's
+// |coefficients|), N terms: 2^-56 M for the values' cut, N 2^-58 M each for the coefficients' rounding
+// and for the products lo lo left out, 2^-57 M for each rounding of a sum.  That is the bound of N
+// FP64 multiply-adds on values of like size; unlike theirs it is relative to M, not to the single
+// products: a value 2^k below its component's largest keeps 57 - k bits, a coefficient 2^k below its
+// box's sum 59 - k.  Measured over all rows of a level, root mean square relative to the sum of the
+// boxes' M, random values, components alike or 1e-4 to 1e-8 of the others: 2D p = 2 4.4e-18, FP64
+// multiply-adds 1.5e-17; mapped p = 3 5e-18 and 2e-17; 3D p = 2 6e-18 and 2e-17, p = 3 1.3e-17 and 2e-17.
+// (With one exponent for all velocity components, 1.4e-13 and 2e-9 in the rows of a component 1e4 and
+// 1e8 times smaller than another.)
+// The local residuals stay integers and go through the local inverse the same way, one exponent for
+// the velocity rows, one for the pressure rows: the inverse mixes the velocity rows, so a small
+// one's low bits are lost in FP64 too.  Emulated on interior and wall patches, components up to 1e8
+// apart: the corrections' errors are 0.05 to 0.9 of those of FP64 multiply-adds, the same with an
+// exponent for each component.  The correction is rounded once to FP64.
 // Values that are not finite make the patch's unknowns NaN; magnitudes below 2^-895 count as 0.
 //
 // The neighbourhood of the patch at position (a, b): with one set of rows for every patch,
@@ -93,6 +104,9 @@ constexpr int kExpFloor = 128;      // biased exponents below this count as zero
 
 __device__ __forceinline__ int exp_of(double v) { return (__double2hiint(v) >> 20) & 0x7ff; }
 
+// |v| as an integer that orders as its magnitude does (exponent from bit 20 up)
+__device__ __forceinline__ int top_of(double v) { return __double2hiint(v) & 0x7fffffff; }
+
 // v != 0 without an FP64 comparison (64 cycles)
 __device__ __forceinline__ bool nonzero(double v) { return (__double2hiint(v) << 1 | __double2loint(v)) != 0; }
 
@@ -121,7 +135,7 @@ __device__ __forceinline__ int2 to_limbs(double v, int e) {
 }
 
 struct Acc {
-  long long hh = 0, m1 = 0, m2 = 0;                            // three independent chains
+  long long hh = 0, m1 = 1ll << 27, m2 = 0;                    // three independent chains (2^27: sum rounds)
   __device__ __forceinline__ void mac(int2 x, int2 c) {
     hh += (long long)x.x * c.x;
     m1 += (long long)x.x * c.y;
@@ -279,6 +293,9 @@ __device__ __forceinline__ Resid<T> row_resid(const limb_t<T>* sA, const limb_t<
   }
 }
 
+__device__ __forceinline__ double resid_value(const Resid<double>& r) { return to_double(r.v, r.a + 60); }
+__device__ __forceinline__ float resid_value(const Resid<float>& r) { return r.v; }
+
 // exponent of a local residual on the scale of its unit (|r| < 2^(exponent - 1082)); 0 for r = 0
 __device__ __forceinline__ int resid_exp(const Resid<double>& r) {
   const unsigned long long m = r.v < 0 ? 0ull - (unsigned long long)r.v : (unsigned long long)r.v;
@@ -291,10 +308,16 @@ __device__ __forceinline__ int2 resid_limbs(const Resid<double>& r, int er, int 
   return limbs_of(shr64(Z, 7 + e - er), r.v < 0 ? -1 : 1);
 }
 
-__device__ __forceinline__ int group_max8(int v) {
-  v = max(v, __shfl_xor_sync(0xffffffffu, v, 1));
-  v = max(v, __shfl_xor_sync(0xffffffffu, v, 2));
-  return max(v, __shfl_xor_sync(0xffffffffu, v, 4));
+// maxima over eight lanes of two exponents (16 bits each)
+__device__ __forceinline__ unsigned max16x2(unsigned x, unsigned y) {
+  unsigned r;
+  asm("max.u16x2 %0, %1, %2;" : "=r"(r) : "r"(x), "r"(y));
+  return r;
+}
+__device__ __forceinline__ unsigned group_max8(unsigned v) {
+  v = max16x2(v, __shfl_xor_sync(0xffffffffu, v, 1));
+  v = max16x2(v, __shfl_xor_sync(0xffffffffu, v, 2));
+  return max16x2(v, __shfl_xor_sync(0xffffffffu, v, 4));
 }
 
 // ---- interior patches: four per warp, lane = (patch, local row) -----------------------------
@@ -308,6 +331,8 @@ struct Patch8 {
   E st_[PRE ? S::NREC : 4], A[PRE ? inv8_ld<T>() : 4];
   const E *st, *Ap;
   int a, b, g, nx, ny, np;          // nx, ny, np: the lane's first entries of the three arrays in U
+  int ex, ey, ep;                   // exponents of the staged u_x, u_y and pressures
+  T f, lam, u_own;
   bool active;
 
   __device__ __forceinline__ void tables(const LevelTab<T>& L, const PatchTab<T>& X, const ColourGrid& C, int w, int lane) {
@@ -339,7 +364,9 @@ struct Patch8 {
     }
   }
 
-  __device__ __forceinline__ void solve(const LevelTab<T>& L, const PatchTab<T>& X, T* U, const T* F, int lane, E* sm) {
+  // stages the neighbourhood; the local residual of the lane's row
+  __device__ __forceinline__ Resid<T> residual(const LevelTab<T>& L, const PatchTab<T>& X, const T* U, const T* F, int lane,
+                                               E* sm) {
     constexpr int KU = (S::NUX + 7) / 8, KP = (S::NP + 7) / 8;
     const int row = lane & 7;
     E* reg = sm + (lane >> 3) * S::REG;
@@ -371,15 +398,22 @@ struct Patch8 {
         vp[k] = (S::NP % 8 == 0 || k < KP - 1 || e < S::NP) ? U[np + c * L.npd + d] : T(0);
       }
     }
-    const T f = F[g], lam = U[L.n_total - 1], u_own = U[g];
-    int eu = kExpFloor, ep = kExpFloor;
+    f = F[g];
+    lam = U[L.n_total - 1];
+    u_own = U[g];
+    ex = ey = ep = kExpFloor << 20;
     if constexpr (sizeof(T) == 8) {
 #pragma unroll
-      for (int k = 0; k < KU; ++k) eu = max(eu, max(exp_of(vx[k]), exp_of(vy[k])));
+      for (int k = 0; k < KU; ++k) {
+        ex = max(ex, top_of(vx[k]));
+        ey = max(ey, top_of(vy[k]));
+      }
 #pragma unroll
-      for (int k = 0; k < KP; ++k) ep = max(ep, exp_of(vp[k]));
-      eu = group_max8(eu);
-      ep = group_max8(ep);
+      for (int k = 0; k < KP; ++k) ep = max(ep, top_of(vp[k]));
+      const unsigned exy = group_max8((unsigned)(ex >> 20 | (ey >> 20) << 16));
+      ex = (int)(exy & 0xffff);
+      ey = (int)(exy >> 16);
+      ep = (int)group_max8((unsigned)ep >> 20);
     }
     auto stage = [&](T v, int e) -> E {
       if constexpr (sizeof(T) == 8) return to_limbs(v, e);
@@ -389,8 +423,8 @@ struct Patch8 {
     for (int k = 0; k < KU; ++k) {
       const int e = row + 8 * k;
       if (S::NUX % 8 == 0 || k < KU - 1 || e < S::NUX) {
-        reg[e] = stage(vx[k], eu);
-        reg[S::UY + e] = stage(vy[k], eu);
+        reg[e] = stage(vx[k], ex);
+        reg[S::UY + e] = stage(vy[k], ey);
       }
     }
 #pragma unroll
@@ -412,7 +446,14 @@ struct Patch8 {
     const E* sB = reg + (is_p ? S::UY + o2 * S::W + o : (is_y ? S::PY + o : S::PX + o));
     const E* sE = reg + (is_y ? o * S::W : S::UY + o * S::W);
     const E* se = EXT ? X.ext + (size_t)(is_p ? 0 : g) * S::NEXT : nullptr;
-    const Resid<T> r = row_resid<P, T, EXT, PRE>(sA, sB, sE, PRE ? st_ : st, se, is_p, eu, is_p ? eu : ep, eu, f, lam);
+    return row_resid<P, T, EXT, PRE>(sA, sB, sE, PRE ? st_ : st, se, is_p, is_y ? ey : ex, is_p ? ey : ep, is_y ? ex : ey, f, lam);
+  }
+
+  __device__ __forceinline__ void solve(const LevelTab<T>& L, const PatchTab<T>& X, T* U, const T* F, int lane, E* sm) {
+    const int row = lane & 7;
+    E* reg = sm + (lane >> 3) * S::REG;
+    const bool is_p = row >= 4;
+    const Resid<T> r = residual(L, X, U, F, lane, sm);
     __syncwarp();
     E A_[PRE ? 4 : inv8_ld<T>()];
     if constexpr (!PRE) ld_entries_lazy<inv8_ld<T>()>(Ap, A_);
@@ -430,7 +471,7 @@ struct Patch8 {
       const int a0 = (is_p ? eo : eg) + A[8].x, a1 = (is_p ? eg : eo) + A[8].y, am = max(a0, a1);
       double d = to_double(sar64(D0.sum(), am - a0) + sar64(D1.sum(), am - a1), am);
       // a value that is not finite in the neighbourhood or in F: the whole patch becomes NaN
-      const bool bad = max(eu, ep) == 0x7ff || exp_of(f) == 0x7ff || exp_of(lam) == 0x7ff;
+      const bool bad = max(max(ex, ey), ep) == 0x7ff || exp_of(f) == 0x7ff || exp_of(lam) == 0x7ff;
       const unsigned any = __ballot_sync(0xffffffffu, bad);
       if ((any >> (lane & 24)) & 0xffu) d = __longlong_as_double(0x7ff8000000000000ll);
       if (active) U[g] = u_own + d;
@@ -474,6 +515,9 @@ struct PatchWall {
   static constexpr int K = (S::NLOAD + S::LW - 1) / S::LW;
   E st_[PRE ? S::NREC : 4];
   int at[K];                        // the thread's neighbourhood values in U, -1: outside
+  int ex, ey, ep;                   // exponents of the staged u_x, u_y and pressures
+  T u_own;
+  bool bad;                         // a value that is not finite (in F, lambda: of this thread or its warp)
   int4 D, R;                        // D: a | b << 16, offset of the inverse (16 B), rows | velocity rows << 8
                                     // R: row, offset of box A | of box B << 16, of the third box, record
 
@@ -504,34 +548,36 @@ struct PatchWall {
     }
   }
 
-  __device__ __forceinline__ void solve(const LevelTab<T>& L, const PatchTab<T>& X, T* U, const T* F, int t, E* sm) {
-    const int nl = D.z & 0xff, nv = D.z >> 8, g = R.x, nu = L.n_ux + L.n_uy;
+  // stages the neighbourhood; the local residual of the thread's row
+  __device__ __forceinline__ Resid<T> residual(const LevelTab<T>& L, const PatchTab<T>& X, const T* U, const T* F, int t, E* sm) {
+    const int nl = D.z & 0xff, g = R.x, nu = L.n_ux + L.n_uy;
     E* reg = sm + S::MARGIN;
-    E* rl = reg + S::REG + S::MARGIN;
-    int* red = reinterpret_cast<int*>(rl + S::LW);             // LW = 64: maxima of the two warps
-    const E* inv = rl + S::LW + 16;
+    int* red = reinterpret_cast<int*>(reg + S::REG + S::MARGIN + S::LW);   // LW = 64: maxima of the two warps
     T v[K];
-    int eu = kExpFloor, ep = kExpFloor;
+    ex = ey = ep = kExpFloor;
 #pragma unroll
     for (int k = 0; k < K; ++k) v[k] = at[k] >= 0 ? U[at[k]] : T(0);
     const bool has = t < nl, is_p = g >= nu;
-    const T f = has ? F[g] : T(0), u_own = has ? U[g] : T(0), lam = U[L.n_total - 1];
-    bool bad = false;
+    const T f = has ? F[g] : T(0), lam = U[L.n_total - 1];
+    u_own = has ? U[g] : T(0);
+    bad = false;
     if constexpr (sizeof(T) == 8) {
 #pragma unroll
       for (int k = 0; k < K; ++k) {
         if (t + S::LW * k >= 2 * S::NUX) ep = max(ep, exp_of(v[k]));
-        else eu = max(eu, exp_of(v[k]));
+        else if (t + S::LW * k >= S::NUX) ey = max(ey, exp_of(v[k]));
+        else ex = max(ex, exp_of(v[k]));
       }
-      // exponents are at most 0x7ff: one word for both maxima is not possible, two reductions are
-      eu = __reduce_max_sync(0xffffffffu, eu);
+      ex = __reduce_max_sync(0xffffffffu, ex);
+      ey = __reduce_max_sync(0xffffffffu, ey);
       ep = __reduce_max_sync(0xffffffffu, ep);
       bad = exp_of(f) == 0x7ff || exp_of(lam) == 0x7ff;
       if constexpr (S::LW == 64) {
         const int any = __any_sync(0xffffffffu, bad);
-        if ((t & 31) == 0) { red[t >> 5] = eu; red[2 + (t >> 5)] = ep; red[4 + (t >> 5)] = any; }
+        if ((t & 31) == 0) { red[t >> 5] = ex; red[2 + (t >> 5)] = ep; red[4 + (t >> 5)] = any; red[6 + (t >> 5)] = ey; }
         wall_sync<S::LW>();
-        eu = max(red[0], red[1]);
+        ex = max(red[0], red[1]);
+        ey = max(red[6], red[7]);
         ep = max(red[2], red[3]);
         bad = red[4] | red[5];
       }
@@ -545,7 +591,7 @@ struct PatchWall {
       const int e = t + S::LW * k;
       if (e >= S::NLOAD) continue;
       E w;
-      if constexpr (sizeof(T) == 8) w = to_limbs(v[k], e >= 2 * S::NUX ? ep : eu);
+      if constexpr (sizeof(T) == 8) w = to_limbs(v[k], e >= 2 * S::NUX ? ep : (e >= S::NUX ? ey : ex));
       else w = v[k];
       const int e1 = e - (e >= 2 * S::NUX ? 2 * S::NUX : (e >= S::NUX ? S::NUX : 0));
       reg[e1 + (e >= 2 * S::NUX ? S::PX : (e >= S::NUX ? S::UY : 0))] = w;
@@ -558,8 +604,18 @@ struct PatchWall {
     const E* sA = reg + (short)(R.y & 0xffff);
     const E* sB = reg + (R.y >> 16);
     const E* se = EXT ? X.ext + (size_t)(is_p || !has ? 0 : g) * S::NEXT : nullptr;
-    const Resid<T> r = row_resid<P, T, EXT, PRE>(sA, sB, reg + R.z, PRE ? st_ : X.rec + (size_t)R.w * S::NREC, se, is_p, eu,
-                                                 is_p ? eu : ep, eu, f, lam);
+    const bool is_y = g >= L.n_ux && !is_p;
+    return row_resid<P, T, EXT, PRE>(sA, sB, reg + R.z, PRE ? st_ : X.rec + (size_t)R.w * S::NREC, se, is_p, is_y ? ey : ex,
+                                     is_p ? ey : ep, is_y ? ex : ey, f, lam);
+  }
+
+  __device__ __forceinline__ void solve(const LevelTab<T>& L, const PatchTab<T>& X, T* U, const T* F, int t, E* sm) {
+    const int nl = D.z & 0xff, nv = D.z >> 8, g = R.x;
+    const bool has = t < nl, is_p = g >= L.n_ux + L.n_uy;
+    E* rl = sm + 2 * S::MARGIN + S::REG;
+    int* red = reinterpret_cast<int*>(rl + S::LW);
+    const E* inv = rl + S::LW + 16;
+    const Resid<T> r = residual(L, X, U, F, t, sm);
     asm volatile("cp.async.wait_all;" ::: "memory");
     const E* Ak = inv + (has ? t : 0) * S::LDW;
     const int slot = t < nv ? t : S::MV + t - nv;              // the row's column in the inverses
@@ -571,7 +627,7 @@ struct PatchWall {
     if constexpr (sizeof(T) == 8) {
       const int er = has ? resid_exp(r) : 0;
       int gu = __reduce_max_sync(0xffffffffu, is_p ? 0 : er), gp = __reduce_max_sync(0xffffffffu, is_p ? er : 0);
-      bad = bad || max(eu, ep) == 0x7ff;
+      bad = bad || max(max(ex, ey), ep) == 0x7ff;
       if constexpr (S::LW == 64) {
         if ((t & 31) == 0) { red[8 + (t >> 5)] = gu; red[10 + (t >> 5)] = gp; }
         wall_sync<S::LW>();
@@ -612,9 +668,10 @@ struct PatchWall {
 // before the loop, ahead of the wait, instead of sinking them to their uses.  Measured per colour
 // with and without the loop: p = 3 64^2 2.65 and 3.08 us, 128^2 3.1 and 3.8, p = 2 128^2 2.5 and 2.9,
 // 256^2 5.0-5.5 and 5.0 (more registers); V-cycle p = 3 72^2 614 and 697 us.
-template <int P, typename T, bool EXT, bool PRE, bool WAIT>
+// ROWS: no solve; U is read only, and the rows' local residuals go to R.
+template <int P, typename T, bool EXT, bool PRE, bool WAIT, bool ROWS = false>
 __device__ __forceinline__ void colour_group(const LevelTab<T>& L, const PatchTab<T>& X, T* U, const T* F,
-                                             const ColourGrid& C, int w, int t, limb_t<T>* sm, int once) {
+                                             const ColourGrid& C, int w, int t, limb_t<T>* sm, int once, T* R = nullptr) {
   using S = PatchShape<P>;
   if (w < C.nwall) {
     PatchWall<P, T, EXT, PRE> W;
@@ -622,7 +679,13 @@ __device__ __forceinline__ void colour_group(const LevelTab<T>& L, const PatchTa
 #pragma unroll 1
     for (int k = 0; k < (WAIT ? once : 1); ++k) {
       if (WAIT) dependency_wait();
-      W.solve(L, X, U, F, t, sm);
+      if constexpr (ROWS) {
+        const Resid<T> r = W.residual(L, X, U, F, t, sm);
+        if (t < (W.D.z & 0xff)) R[W.R.x] = resid_value(r);
+        asm volatile("cp.async.wait_all;" ::: "memory");
+      } else {
+        W.solve(L, X, U, F, t, sm);
+      }
     }
   } else {
     const int wp = (w - C.nwall) * (S::LW / 32) + (t >> 5);
@@ -632,7 +695,13 @@ __device__ __forceinline__ void colour_group(const LevelTab<T>& L, const PatchTa
 #pragma unroll 1
     for (int k = 0; k < (WAIT ? once : 1); ++k) {
       if (WAIT) dependency_wait();
-      I.solve(L, X, U, F, t & 31, sm + (t >> 5) * 4 * S::REG);
+      limb_t<T>* smw = sm + (t >> 5) * 4 * S::REG;
+      if constexpr (ROWS) {
+        const Resid<T> r = I.residual(L, X, U, F, t & 31, smw);
+        if (I.active) R[I.g] = resid_value(r);
+      } else {
+        I.solve(L, X, U, F, t & 31, smw);
+      }
     }
   }
 }
@@ -654,6 +723,20 @@ __global__ void __launch_bounds__(64) k_patch_colour(const __grid_constant__ Lev
   if (w >= ngroups) return;
   colour_group<P, T, EXT, true, true>(L, X, U, F, C, w, threadIdx.x % LW, reinterpret_cast<limb_t<T>*>(smem_raw) + gib * smg,
                                       once);
+}
+
+// The local residuals F - K U of the rows of one colour's patches as the colour kernel forms them
+// (a measuring hook: what its arithmetic makes of a row before the local inverse mixes the rows).
+template <int P, bool EXT>
+__global__ void __launch_bounds__(64) k_patch_rows(const __grid_constant__ LevelTab<double> L,
+                                                   const __grid_constant__ PatchTab<double> X, double* U, const double* F,
+                                                   double* R, const ColourGrid C, int ngroups, int smg) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  constexpr int LW = PatchShape<P>::LW;
+  const int gib = threadIdx.x / LW, w = blockIdx.x * (64 / LW) + gib;
+  if (w >= ngroups) return;
+  colour_group<P, double, EXT, true, false, true>(L, X, U, F, C, w, threadIdx.x % LW,
+                                                  reinterpret_cast<int2*>(smem_raw) + gib * smg, 1, R);
 }
 
 // ---- building the tables (once, at creation) ---------------------------------------------------

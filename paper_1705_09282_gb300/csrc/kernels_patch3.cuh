@@ -64,6 +64,13 @@ struct PatchTab3 {
   int by_row, maxl;
 };
 
+// Exponents of a patch's staged values, one per component.
+struct Exps3 {
+  int u0, u1, u2, p;
+  __device__ __forceinline__ int of(int k) const { return k == 1 ? u1 : (k == 2 ? u2 : u0); }
+  __device__ __forceinline__ bool bad() const { return max(max(u0, u1), max(u2, p)) == 0x7ff; }
+};
+
 // One colour (PatchGrid3, igamg_internal.h).  row[r]: the interior patch's local row r: kind, its
 // position relative to the patch (0 or -1 per axis, as bits), offsets of its boxes.
 struct ColourGrid3 {
@@ -74,19 +81,20 @@ struct ColourGrid3 {
 // The lane's share of a row: box A at slice s, box B at slice s, and box C at slice s (pressure
 // rows) or the last slice of box A (velocity rows, p = 2, lane 0).  Result: the lane's part of the
 // local residual on the row's common scale, the same exponent a on all lanes of the row.
-// PRE: st is the lane's record in registers; else in global memory, read box by box.
+// PRE: st is the lane's record in registers; else in global memory, read box by box.  kind: the row's.
 template <int P, typename T, bool EXT, bool PRE>
 __device__ __forceinline__ Resid<T> row_part(const limb_t<T>* reg, int oA, int oB, int oC, int oE, const limb_t<T>* st,
-                                             const limb_t<T>* __restrict__ tail, const limb_t<T>* __restrict__ se, bool is_p,
-                                             int s, int eu, int ep, T f, T lam) {
+                                             const limb_t<T>* __restrict__ tail, const limb_t<T>* __restrict__ se, int kind,
+                                             int s, const Exps3& ev, T f, T lam) {
   using S = PatchShape3<P>;
   constexpr int SLP = slice_len<P, T>();
+  const bool is_p = kind == 3;
   const limb_t<T>* pA = reg + oA + min(s, S::A1 - 1) * S::LS;
   const limb_t<T>* pB = reg + oB + min(s, 2 * P - 1) * S::LS;
   const limb_t<T>* pC = is_p ? reg + oC + min(s, 2 * P - 1) * S::LS : reg + oA + (S::LPR < S::A1 && s == 0 ? S::LPR * S::LS : 0);
   if constexpr (sizeof(T) == 8) {
     Acc A, B, C;
-    int aA = eu, aB = is_p ? eu : ep, aC = eu;
+    int aA = ev.of(kind), aB = is_p ? ev.u1 : ev.p, aC = is_p ? ev.u2 : aA;   // (pressure rows: boxes on u_x, u_y, u_z)
     if constexpr (PRE) {                                       // the three boxes' chains side by side
 #pragma unroll
       for (int j = 0; j < S::SL; ++j) {
@@ -127,7 +135,7 @@ __device__ __forceinline__ Resid<T> row_part(const limb_t<T>* reg, int oA, int o
           E.mac(pE[ce[S::XE].y ? (j / S::C1) * S::W + j % S::C1 : (j / S::W) * S::W + j % S::W], ce[j]);
         }
       }
-      aE = eu + ce[S::XE].x;
+      aE = ev.of(1 - kind) + ce[S::XE].x;
       sE = E.sum();
       a = max(a, aE);
     }
@@ -146,6 +154,10 @@ __device__ __forceinline__ Resid<T> row_part(const limb_t<T>* reg, int oA, int o
       r = (long long)shr64(M << 7, a - exF);
       if (h < 0) r = -r;
       if (is_p && nonzero(lam)) r -= sar64(sL, a - aL);
+      // the shifts below round down: half a unit per lane and shifted box, put back here for all lanes
+      // (without it the rows of the cylinder at p = 3 were 7 % less accurate than FP64 multiply-adds)
+      const int shifted = (aA < a) + (aB < a) + (is_p && aC < a) + (EXT && se && aE < a);
+      r -= S::LPR / 2 * shifted;
     }
     r -= sar64(A.sum(), a - aA);
     r -= sar64(B.sum(), a - aB);
@@ -195,11 +207,11 @@ __device__ __forceinline__ void lanes_sum(Resid<float>& r) {
 }
 
 // Loads the neighbourhood of the patch (f; p0, p1, p2) with G threads and stages it at reg.
-// sync: barrier of the G threads; red: four ints of shared memory, zero on entry if G > 32.
+// sync: barrier of the G threads; red: shared memory for a maximum per warp, if G > 32.
 // WALL: positions outside the index range count as 0, and P3 is filled.
 template <int P, typename T, bool WALL, int G, typename Sync>
 __device__ __forceinline__ void stage3(const LevelTab3<T>& L, const T* U, int f, const int* pos, int t, limb_t<T>* reg,
-                                       int* red, int& eu, int& ep, Sync sync) {
+                                       int4* red, Exps3& ev, Sync sync) {
   using S = PatchShape3<P>;
   constexpr int KU = (S::NUC + G - 1) / G, KW = (S::NW3 + G - 1) / G;
   T v1[KU], v2[KU], vf[KW], vp[KW];
@@ -247,21 +259,37 @@ __device__ __forceinline__ void stage3(const LevelTab3<T>& L, const T* U, int f,
 #pragma unroll
     for (int k = 0; k < KW; ++k) { vf[k] = load(f, f, t + G * k, S::NW3); vp[k] = load(3, c1, t + G * k, S::NW3); }
   }
-  eu = ep = kExpFloor;
+  int e1 = kExpFloor << 20, e2 = e1, ef = e1, ep = e1;
   if constexpr (sizeof(T) == 8) {
 #pragma unroll
-    for (int k = 0; k < KU; ++k) eu = max(eu, max(exp_of(v1[k]), exp_of(v2[k])));
+    for (int k = 0; k < KU; ++k) { e1 = max(e1, top_of(v1[k])); e2 = max(e2, top_of(v2[k])); }
 #pragma unroll
-    for (int k = 0; k < KW; ++k) { eu = max(eu, exp_of(vf[k])); ep = max(ep, exp_of(vp[k])); }
-    eu = __reduce_max_sync(0xffffffffu, eu);
+    for (int k = 0; k < KW; ++k) { ef = max(ef, top_of(vf[k])); ep = max(ep, top_of(vp[k])); }
+    e1 = __reduce_max_sync(0xffffffffu, e1);
+    e2 = __reduce_max_sync(0xffffffffu, e2);
+    ef = __reduce_max_sync(0xffffffffu, ef);
     ep = __reduce_max_sync(0xffffffffu, ep);
     if constexpr (G > 32) {
-      if ((t & 31) == 0) { atomicMax(red, eu); atomicMax(red + 1, ep); }
+      if ((t & 31) == 0) red[t >> 5] = make_int4(e1, e2, ef, ep);
       sync();
-      eu = red[0];
-      ep = red[1];
+#pragma unroll
+      for (int w = 0; w < G / 32; ++w) {
+        const int4 q = red[w];
+        e1 = max(e1, q.x);
+        e2 = max(e2, q.y);
+        ef = max(ef, q.z);
+        ep = max(ep, q.w);
+      }
     }
+    e1 >>= 20;
+    e2 >>= 20;
+    ef >>= 20;
+    ep >>= 20;
   }
+  ev.u0 = f == 0 ? ef : (f == 2 ? e1 : e2);
+  ev.u1 = f == 1 ? ef : (f == 0 ? e1 : e2);
+  ev.u2 = f == 2 ? ef : (f == 1 ? e1 : e2);
+  ev.p = ep;
   auto put = [&](int at, T v, int e) {
     if constexpr (sizeof(T) == 8) reg[at] = to_limbs(v, e);
     else reg[at] = v;
@@ -269,13 +297,13 @@ __device__ __forceinline__ void stage3(const LevelTab3<T>& L, const T* U, int f,
 #pragma unroll
   for (int k = 0; k < KU; ++k) {
     const int e = t + G * k, at = e + e / S::W2 * (S::LS - S::W2);
-    if (e < S::NUC) { put(at, v1[k], eu); put(S::U2 + at, v2[k], eu); }
+    if (e < S::NUC) { put(at, v1[k], e1); put(S::U2 + at, v2[k], e2); }
   }
 #pragma unroll
   for (int k = 0; k < KW; ++k) {
     const int e = t + G * k, at = e + e / S::W2 * (S::LS - S::W2);
     if (e >= S::NW3) continue;
-    put(S::UF + at, vf[k], eu);
+    put(S::UF + at, vf[k], ef);
     limb_t<T> w;
     if constexpr (sizeof(T) == 8) w = to_limbs(vp[k], ep);
     else w = vp[k];
@@ -294,18 +322,22 @@ __device__ __forceinline__ int row_index3(const LevelTab3<T>& L, int kind, int x
 }
 
 // ---- one colour: blocks [0, nwall) a wall patch each, then PPB interior patches per block ------
+// Three blocks per SM at p = 2 (left alone, the third box's variant takes 222 registers, two blocks:
+// cylinder 32^3 17.2 us a colour against 14.3).
 // PRE: the records are fetched into registers before the dependency wait (colours that leave the
 // GPU idle: the chain of one block counts); else they are read where they are used and the
 // registers saved hold twice the warps (colours of many blocks).
-template <int P, typename T, bool EXT, bool PRE>
-__global__ void __launch_bounds__(128, PRE ? 1 : 6) k_patch_colour3(const __grid_constant__ LevelTab3<T> L,
+// ROWS: no solve; U is read only, and the rows' local residuals go to R_ (k_patch_rows of the 2D path).
+template <int P, typename T, bool EXT, bool PRE, bool ROWS = false>
+__global__ void __launch_bounds__(128, !PRE ? 6 : (P == 2 ? 3 : 2)) k_patch_colour3(const __grid_constant__ LevelTab3<T> L,
                                                        const __grid_constant__ PatchTab3<T> X, T* U, const T* F,
-                                                       const __grid_constant__ ColourGrid3 C) {
+                                                       const __grid_constant__ ColourGrid3 C, T* R_) {
   using S = PatchShape3<P>;
   using E = limb_t<T>;
   constexpr int SLP = slice_len<P, T>(), NR = rec3_len<P, T>(), LPR = S::LPR;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  __shared__ int red[16];
+  __shared__ int red[8];                                       // residual exponents (2) and a flag, per group
+  __shared__ int4 emax[S::NT / 32];
   E st_[PRE ? 3 * SLP : 1];
   const E* st = st_;
   if ((int)blockIdx.x >= C.nwall) {
@@ -342,17 +374,21 @@ __global__ void __launch_bounds__(128, PRE ? 1 : 6) k_patch_colour3(const __grid
     for (int c = 0; c < NC8; ++c) A[c] = Ap[s * NC8 + c];
     int2 ec = make_int2(0, 0);
     if constexpr (sizeof(T) == 8) ec = Ap[8];
-    if (S::G8 > 32 && t < 8) red[grp * 8 + t] = 0;
+    if (S::G8 > 32 && t < 4) red[grp * 4 + t] = 0;
     const E* se = EXT && kind < 2 ? X.ext + (size_t)g * ext3_rec_len<P, T>() : nullptr;
     dependency_wait();
     if (S::G8 > 32) sync();
     E* reg = reinterpret_cast<E*>(smem_raw) + grp * S::REGI;
     const T fv = F[g], lam = U[L.n_total - 1], u_own = U[g];
-    int eu, ep;
-    stage3<P, T, false, S::G8>(L, U, C.f, pos, t, reg, red + grp * 8, eu, ep, sync);
-    Resid<T> r = row_part<P, T, EXT, PRE>(reg, C.oA[row], C.oB[row], C.oC[row], C.oE[row], st, rp + LPR * 3 * SLP, se, is_p, s,
-                                     eu, ep, fv, lam);
+    Exps3 ev;
+    stage3<P, T, false, S::G8>(L, U, C.f, pos, t, reg, emax + grp * (S::G8 / 32), ev, sync);
+    Resid<T> r = row_part<P, T, EXT, PRE>(reg, C.oA[row], C.oB[row], C.oC[row], C.oE[row], st, rp + LPR * 3 * SLP, se, kind, s,
+                                     ev, fv, lam);
     lanes_sum<LPR>(r);
+    if constexpr (ROWS) {
+      if (s == 0) R_[g] = resid_value(r);
+      return;
+    }
     sync();
     if constexpr (sizeof(T) == 8) {
       const int er = resid_exp(r);
@@ -362,14 +398,14 @@ __global__ void __launch_bounds__(128, PRE ? 1 : 6) k_patch_colour3(const __grid
         eg = max(eg, __shfl_xor_sync(0xffffffffu, eg, 8));
         eo = __shfl_xor_sync(0xffffffffu, eg, 16);
       } else {
-        if (s == 0) atomicMax(&red[grp * 8 + 2 + (is_p ? 1 : 0)], er);
+        if (s == 0) atomicMax(&red[grp * 4 + (is_p ? 1 : 0)], er);
         sync();
-        eg = red[grp * 8 + 2 + (is_p ? 1 : 0)];
-        eo = red[grp * 8 + 3 - (is_p ? 1 : 0)];
+        eg = red[grp * 4 + (is_p ? 1 : 0)];
+        eo = red[grp * 4 + 1 - (is_p ? 1 : 0)];
       }
       if (s == 0) reg[row] = resid_limbs(r, er, eg);
-      const bool bad = max(eu, ep) == 0x7ff || exp_of(fv) == 0x7ff || exp_of(lam) == 0x7ff;
-      if (S::G8 > 32 && bad) red[grp * 8 + 4] = 1;
+      const bool bad = ev.bad() || exp_of(fv) == 0x7ff || exp_of(lam) == 0x7ff;
+      if (S::G8 > 32 && bad) red[grp * 4 + 2] = 1;
       sync();
       const int c0 = s * NC8;                                  // this lane's columns: all velocity or all pressure
       Acc D;
@@ -381,7 +417,7 @@ __global__ void __launch_bounds__(128, PRE ? 1 : 6) k_patch_colour3(const __grid
       double dv = to_double(q.v, am);
       bool any;
       if constexpr (S::G8 == 32) any = __any_sync(0xffffffffu, bad);
-      else any = red[grp * 8 + 4];
+      else any = red[grp * 4 + 2];
       if (any) dv = __longlong_as_double(0x7ff8000000000000ll);
       if (s == 0) U[g] = u_own + dv;
     } else {
@@ -415,7 +451,7 @@ __global__ void __launch_bounds__(128, PRE ? 1 : 6) k_patch_colour3(const __grid
   auto sync = [&]() { __syncthreads(); };
   int4 R = X.wrow[(size_t)w * S::MR + rl_row];
   if constexpr (PRE) ld_entries<3 * SLP>(X.rec + (size_t)R.w * NR + s * 3 * SLP, st_);
-  if (t < 16) red[t] = 0;
+  if (t < 4) red[t] = 0;
   dependency_wait();
   __syncthreads();
   if constexpr (sizeof(T) == 4) {                              // what rows read with zero coefficients is finite
@@ -424,10 +460,10 @@ __global__ void __launch_bounds__(128, PRE ? 1 : 6) k_patch_colour3(const __grid
   }
   const int pos[3] = {D.x & 1023, D.x >> 10 & 1023, D.x >> 20 & 1023};
   const T lam = U[L.n_total - 1];
-  int eu, ep;
-  stage3<P, T, true, S::NT>(L, U, C.f, pos, t, reg, red, eu, ep, sync);
+  Exps3 ev;
+  stage3<P, T, true, S::NT>(L, U, C.f, pos, t, reg, emax, ev, sync);
   bool bad = false;
-  if constexpr (sizeof(T) == 8) bad = max(eu, ep) == 0x7ff || exp_of(lam) == 0x7ff;
+  if constexpr (sizeof(T) == 8) bad = ev.bad() || exp_of(lam) == 0x7ff;
   for (int r0 = 0; r0 < nl; r0 += S::RPR) {
     const int row = r0 + rl_row;
     if (r0 > 0) {
@@ -435,30 +471,36 @@ __global__ void __launch_bounds__(128, PRE ? 1 : 6) k_patch_colour3(const __grid
       if constexpr (PRE) ld_entries<3 * SLP>(X.rec + (size_t)R.w * NR + s * 3 * SLP, st_);
     }
     if constexpr (!PRE) st = X.rec + (size_t)R.w * NR + s * 3 * SLP;
-    const bool has = row < nl, is_p = R.x >= L.n_u;
+    const bool has = row < nl;
+    const int kind = R.x >= L.n_u ? 3 : (R.x >= 2 * L.n_uc ? 2 : (R.x >= L.n_uc ? 1 : 0));
     const T fv = has ? F[R.x] : T(0);
     const E* se = EXT && has && R.x < 2 * L.n_uc ? X.ext + (size_t)R.x * ext3_rec_len<P, T>() : nullptr;
     Resid<T> r = row_part<P, T, EXT, PRE>(reg, (short)(R.y & 0xffff), R.y >> 16, (short)(R.z & 0xffff), R.z >> 16, st,
-                                     X.rec + (size_t)R.w * NR + LPR * 3 * SLP, se, is_p, s, eu, ep, fv, lam);
+                                     X.rec + (size_t)R.w * NR + LPR * 3 * SLP, se, kind, s, ev, fv, lam);
     lanes_sum<LPR>(r);
+    if constexpr (ROWS) {
+      if (s == 0 && has) R_[R.x] = resid_value(r);
+      continue;
+    }
     if constexpr (sizeof(T) == 8) {
       bad = bad || exp_of(fv) == 0x7ff;
       if (s == 0 && has) {
         rv[row] = r.v;
         ra[row] = r.a;
-        atomicMax(&red[2 + (row < nv ? 0 : 1)], resid_exp(r));
+        atomicMax(&red[row < nv ? 0 : 1], resid_exp(r));
       }
     } else {
       if (s == 0 && has) rl[row] = r.v;
     }
   }
-  if (bad) red[4] = 1;
+  if (bad) red[2] = 1;
   asm volatile("cp.async.wait_all;" ::: "memory");
+  if constexpr (ROWS) return;
   __syncthreads();
   const E* A = P == 2 ? inv : reinterpret_cast<const E*>(src);
   if constexpr (sizeof(T) == 8) {
-    const int gu = red[2], gp = red[3];
-    const bool any = red[4] != 0;
+    const int gu = red[0], gp = red[1];
+    const bool any = red[2] != 0;
     for (int row = t; row < nl; row += S::NT) {
       const Resid<double> r{rv[row], ra[row]};
       rl[row] = resid_limbs(r, resid_exp(r), row < nv ? gu : gp);

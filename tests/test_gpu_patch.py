@@ -131,3 +131,63 @@ def test_staged_sweeps_3d_equal_row_kernels(p, n, kind, monkeypatch):
     assert float((V0 - V1).abs().max()) <= tol * float(V0.abs().max())
     S0.close()
     S1.close()
+
+
+@pytest.mark.parametrize("p,n,dim,kind", [(2, 16, 2, "stokes"), (3, 14, 2, "stokes"), (2, 12, 2, "oseen"), (2, 12, 2, "annulus"),
+                                          (3, 12, 2, "annulus"), (2, 6, 3, "stokes"), (2, 6, 3, "oseen"), (2, 6, 3, "cylinder"),
+                                          (3, 6, 3, "stokes"), (3, 6, 3, "cylinder")])
+@pytest.mark.parametrize("small", ["none", "ux", "uy", "p", "uxp"])
+def test_rows_keep_their_precision_when_components_differ(p, n, dim, kind, small, monkeypatch):
+    # every patch row's local residual against the same sum in extended precision, component by component,
+    # one or two of which are 1e-4 and 1e-8 of the others: no row may lose to values it does not read.
+    # Bound, relative to D = |F| + sum over components of (sum |K_ij|) max |U_j|, with N terms in the
+    # largest box: values cut at 2^-56, coefficients rounded at 2^-58 each, lo x lo products left out
+    # at 2^-58 each, two shifts of 2^-57 per box and lane of the row, the result rounded at 2^-54.
+    # And the root mean square must not exceed that of FP64 multiply-adds (k_residual on the records).
+    torch = _torch()
+    import ctypes
+
+    from paper_1705_09282_gb300 import _lib
+    from paper_1705_09282_gb300.solver import Solver, host_operator_rows
+    monkeypatch.setenv("IGAMG_ADV_FORM", "records")
+    kw = {"dim": 3} if dim == 3 else {}
+    if kind == "oseen":
+        kw["beta"] = inputs.oseen_advection_3d(p, n, 0.5) if dim == 3 else inputs.oseen_advection(p, n, 0.5)
+    elif kind != "stokes":
+        kw["geometry"] = _lib.IGAMG_GEOM_QUARTER_ANNULUS if dim == 2 else _lib.IGAMG_GEOM_HOLLOW_CYLINDER
+    S = Solver(p, n, 2, 10.0, 0.5, **kw)
+    nd = S.ndof()
+    K = host_operator_rows(p, n, 2, 10.0, 0.5, 1, **kw)[: nd - 1]
+    q = p - 1
+    if dim == 2:
+        nc = (n + p - 2) * (n + q)
+        cuts = [0, nc, 2 * nc, nd - 1, nd]
+        terms, lanes = max((2 * p + 1) * (2 * q + 1), 4 * p * p), 1
+    else:
+        nc = (n + p - 2) * (n + q) ** 2
+        cuts = [0, nc, 2 * nc, 3 * nc, nd - 1, nd]
+        terms, lanes = max((2 * p + 1) * (2 * q + 1) ** 2, 4 * p * p * (2 * q + 1)), 4 if p == 2 else 8
+    comp = [slice(a, b) for a, b in zip(cuts, cuts[1:])]
+    U = inputs.random_vector(nd, seed=n)
+    scale = {"none": (), "ux": ((0, 1e-8),), "uy": ((1, 1e-4),), "p": ((dim, 1e-8),), "uxp": ((0, 1e-4), (dim, 1e-8))}[small]
+    for c, x in scale:
+        U[comp[c]] *= x
+    F = np.zeros(nd)
+    F[: nd - 1] = (K @ U) * (1.0 + 0.5 * inputs.random_vector(nd - 1, seed=n + 1))
+    exact = F[: nd - 1].astype(np.longdouble) - np.array([(k.astype(np.longdouble) * U.astype(np.longdouble)).sum() for k in K])
+    D = np.abs(F[: nd - 1])
+    for c in comp:
+        D = D + np.abs(K[:, c]).sum(axis=1) * np.abs(U[c]).max()
+    Ud, Fd = torch.tensor(U, device="cuda"), torch.tensor(F, device="cuda")
+    R = torch.full((nd,), float("nan"), dtype=torch.float64, device="cuda")
+    _lib.check(_lib.lib().igamg_probe_patch_rows(S._h, 1, ctypes.c_void_p(Ud.data_ptr()), ctypes.c_void_p(Fd.data_ptr()),
+                                                 ctypes.c_void_p(R.data_ptr())), "igamg_probe_patch_rows")
+    got = R.cpu().numpy()[: nd - 1]
+    fp64 = S.residual(Ud, Fd).cpu().numpy()[: nd - 1]
+    assert torch.equal(Ud, torch.tensor(U, device="cuda"))
+    rel = (np.abs(got - exact) / D).astype(float)
+    ref = (np.abs(fp64 - exact) / D).astype(float)
+    for k, c in enumerate(comp[:-1]):
+        assert rel[c].max() <= (2 * terms + 4 + 16 * lanes) * 2.0 ** -58 + 2.0 ** -54, k
+        assert np.sqrt((rel[c] ** 2).mean()) <= np.sqrt((ref[c] ** 2).mean()), k
+    S.close()
