@@ -28,7 +28,8 @@
 // one's low bits are lost in FP64 too.  Emulated on interior and wall patches, components up to 1e8
 // apart: the corrections' errors are 0.05 to 0.9 of those of FP64 multiply-adds, the same with an
 // exponent for each component.  The correction is rounded once to FP64.
-// Values that are not finite make the patch's unknowns NaN; magnitudes below 2^-895 count as 0.
+// Values that are not finite make the patch's unknowns NaN; where all of a component is below 2^-959 (biased
+// exponent 64) its low bits go, denormals count as 0.
 //
 // The neighbourhood of the patch at position (a, b): with one set of rows for every patch,
 //   UX [2p+1][2p]  u_x at x = a-p .. a+p (outer), y = b-p .. b+p-1
@@ -100,7 +101,7 @@ struct ColourGrid {
   int a0, b0, na, n8, gfirst, wfirst, nwall;
 };
 
-constexpr int kExpFloor = 128;      // biased exponents below this count as zero
+constexpr int kExpFloor = 64;       // least exponent of a group: zeros and denormals (biased exponent 0) shift out
 
 __device__ __forceinline__ int exp_of(double v) { return (__double2hiint(v) >> 20) & 0x7ff; }
 

@@ -191,3 +191,21 @@ def test_rows_keep_their_precision_when_components_differ(p, n, dim, kind, small
         assert rel[c].max() <= (2 * terms + 4 + 16 * lanes) * 2.0 ** -58 + 2.0 ** -54, k
         assert np.sqrt((rel[c] ** 2).mean()) <= np.sqrt((ref[c] ** 2).mean()), k
     S.close()
+
+
+@pytest.mark.parametrize("dim,p,n", [(2, 2, 16), (2, 3, 16), (3, 2, 8)])
+@pytest.mark.parametrize("scale", [2.0 ** -920, 2.0 ** 940])
+def test_staged_sweep_near_the_ends_of_the_exponent_range(dim, p, n, scale):
+    # as test_staged_sweep_at_extreme_scales; the largest value of every component of a neighbourhood stays
+    # above 2^-959 here, below which the staged rows give up low bits
+    torch = _torch()
+    from paper_1705_09282_gb300.solver import Solver
+    S = Solver(p, n, 2, 1.0, 1.0, **({"dim": 3} if dim == 3 else {}))
+    nd = S.ndof()
+    U = torch.tensor(inputs.random_vector(nd, seed=3), device="cuda")
+    F = torch.tensor(inputs.random_vector(nd, seed=4), device="cuda")
+    V, W = U.clone(), U * scale
+    S.smooth(V, F)
+    S.smooth(W, F * scale)
+    assert torch.equal(W, V * scale)
+    S.close()
