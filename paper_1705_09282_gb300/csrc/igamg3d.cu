@@ -209,6 +209,15 @@ struct Typed3 {
   Cluster3Desc<T> cdesc{};
 };
 
+// Most blocks of a colour launch whose records are fetched ahead of the dependency wait (PRE of
+// k_patch_colour3); IGAMG_PRE_BLOCKS, read at creation, takes its place (tests).  us per colour, ahead and
+// in place, FP64: p = 2 Stokes 32^3 (550 to 1150 blocks) 10.2 and 10.0, 48^3 (2500) 25.1 and 20.9, 64^3
+// 52.7 and 40.1; Oseen records 32^3 11.9 and 13.3, 48^3 31.9 and 28.7; cylinder 32^3 14.5 and 15.2, 40^3
+// 24.2 and 21.9; p = 3 Stokes (all below the line) 16^3 29.7 and 31.4, 24^3 26.7 and 31.2, 32^3 33.4 and
+// 36.0.  The line was drawn for FP64; FP32 V-cycles take 2893 and 3044 us at 32^3, 4847 and 5057 at
+// 48^3, 8798 and 9037 at 64^3, so they lose 3 to 4 % above it.
+constexpr int kPreBlocks = 1500;
+
 struct Lev3Common {
   int n_patches = 0, maxl = 0, n_colours = 0, row_slots = 0;
   std::vector<int> colour_off, n8, colour_blk;
@@ -244,6 +253,7 @@ struct igamg3d_handle {
   KrylovWork kw;                    // FGMRES modes
   double* zeros = nullptr;
   double* jt = nullptr;              // mapped domains: J^T at the finest quadrature points
+  int pre_blocks = kPreBlocks;       // IGAMG_PRE_BLOCKS at creation
 };
 
 namespace {
@@ -446,11 +456,6 @@ int do_residual(igamg3d_handle* h, int l, const T* U, const T* F, T* R, double* 
   return launch_check();
 }
 
-// Most blocks of a colour launch whose records are fetched ahead of the dependency wait (PRE of
-// k_patch_colour3).  Measured at p = 2, FP64, per colour: 32^3 (about 500 blocks) 10.3 us ahead, 10.4
-// in place, Oseen records 12.2 and 13.9; 64^3 (3600 blocks) 52.7 and 40.1.
-constexpr int kPreBlocks = 1500;
-
 // One sweep of staged patch solves, one launch per colour, each allowed to fetch its tables while the
 // launch before it runs (programmatic dependent launch, as in the 2D path).
 template <int P, typename T>
@@ -471,7 +476,7 @@ int do_smooth_staged(igamg3d_handle* h, int l, T* U, const T* F, cudaStream_t s)
     const int nb = C.nwall + (C.n8 + S::PPB - 1) / S::PPB;
     if (nb == 0) continue;
     cfg.gridDim = dim3((unsigned)nb);
-    const bool pre = nb <= kPreBlocks;
+    const bool pre = nb <= h->pre_blocks;
     T* const none = nullptr;
     cudaError_t e;
     if (tl.X.ext) e = pre ? cudaLaunchKernelEx(&cfg, k_patch_colour3<P, T, true, true>, tl.L, tl.X, U, F, C, none)
@@ -888,6 +893,7 @@ int h3_create(const igamg_problem* prob, void* cuda_stream, igamg3d_handle** out
   auto* h = new igamg3d_handle();
   h->prob = pr;
   h->stream = (cudaStream_t)cuda_stream;
+  if (const char* e = std::getenv("IGAMG_PRE_BLOCKS")) h->pre_blocks = std::atoi(e);
   std::string err;
   rc = build_hierarchy3(pr, h->host, err);
   if (rc) { set_error(err); delete h; return rc; }

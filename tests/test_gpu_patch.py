@@ -209,3 +209,38 @@ def test_staged_sweep_near_the_ends_of_the_exponent_range(dim, p, n, scale):
     S.smooth(W, F * scale)
     assert torch.equal(W, V * scale)
     S.close()
+
+
+@pytest.mark.parametrize("p,n", [(2, 6), (2, 10), (3, 6)])
+@pytest.mark.parametrize("kind", ["stokes", "oseen", "cylinder", "fp32", "cylinder-fp32"])
+def test_3d_records_read_in_place_equal_records_fetched_ahead(p, n, kind, monkeypatch):
+    # the variant for colours of many blocks, on meshes small enough to run every form: the FP64 rows are
+    # integers, so both variants agree bit for bit (FP32: the tolerance of the sweep against the row kernels)
+    torch = _torch()
+    from paper_1705_09282_gb300 import _lib
+    from paper_1705_09282_gb300.solver import Solver
+    kw = {"dim": 3}
+    if kind == "oseen":
+        kw["beta"] = inputs.oseen_advection_3d(p, n, 0.5)
+    if kind.startswith("cylinder"):
+        kw["geometry"] = _lib.IGAMG_GEOM_HOLLOW_CYLINDER
+    if kind.endswith("fp32"):
+        kw["precision"] = _lib.IGAMG_FP32_IR
+    monkeypatch.setenv("IGAMG_FUSED_LEVELS", "-1")
+    out = []
+    for blocks in ("0", str(1 << 30)):
+        monkeypatch.setenv("IGAMG_PRE_BLOCKS", blocks)
+        S = Solver(p, n, 2, 10.0, 0.5, **kw)
+        F = torch.tensor(inputs.random_vector(S.ndof(), seed=n + 1), device="cuda")
+        if kind.endswith("fp32"):
+            V = S.empty()
+            S.vcycle(V, F)
+        else:
+            V = torch.tensor(inputs.random_vector(S.ndof(), seed=n), device="cuda")
+            S.smooth(V, F, sweeps=2)
+        out.append(V.clone())
+        S.close()
+    if kind.endswith("fp32"):
+        assert float((out[0] - out[1]).abs().max()) <= 5e-5 * float(out[1].abs().max())
+    else:
+        assert torch.equal(out[0], out[1])
