@@ -339,6 +339,15 @@ int dmalloc(igamg_handle* h, void** p, size_t bytes) {
   return IGAMG_OK;
 }
 
+// Frees one of the handle's allocations early.
+template <typename V>
+void dfree(igamg_handle* h, V*& p) {
+  if (!p) return;
+  h->allocs.erase(std::find(h->allocs.begin(), h->allocs.end(), (void*)p));
+  cudaFree((void*)p);
+  p = nullptr;
+}
+
 template <typename V, typename S>
 int upload_as(igamg_handle* h, V** dst, const std::vector<S>& src) {
   std::vector<V> tmp(src.begin(), src.end());
@@ -1693,8 +1702,17 @@ std::vector<double> round_bf16(const std::vector<double>& v) {
   return out;
 }
 
+template <typename Tab, typename H>
+void drop_patch_tab(H* h, Tab& X) {
+  dfree(h, X.rec);
+  dfree(h, X.ext);
+  dfree(h, X.inv8);
+  dfree(h, X.winv);
+}
+
 // The staged patch kernels' records and inverses of level l, made on the device from the uploaded
-// tables (FP64: integer limbs; FP32: the same values, u_y rows with y outer).
+// tables (FP64: integer limbs; FP32: the same values, u_y rows with y outer).  Where memory is short
+// (staged_fits) the level is left to the row kernels: lc.grids is emptied.
 template <int P, typename T>
 int build_patch_tab(igamg_handle* h, int l, TypedLevel<T>& tl) {
   using S = PatchShape<P>;
@@ -1705,6 +1723,14 @@ int build_patch_tab(igamg_handle* h, int l, TypedLevel<T>& tl) {
   PatchGrids G;                    // (offsets of the inverses differ between FP64 limbs and FP32)
   if (!patch_grids(P, lh.sz, lh.pt, L.srow != nullptr, (int)sizeof(E), G)) return IGAMG_EINVAL;
   PatchTab<T>& X = tl.X;
+  const int n8 = std::max(lh.pt.n_cls8, 1), nw = (int)G.wspec.size() / 4;
+  const size_t nrec = L.srow ? (size_t)L.n_total - 1 : 3 * (lh.st.sx.size() / S::RU);
+  const size_t next = L.sext ? (size_t)(L.n_ux + L.n_uy) * S::NEXT : 0;
+  if (!staged_fits((nrec * S::NREC + next + (size_t)n8 * 8 * inv8_ld<T>()) * sizeof(E) + (size_t)std::max(G.winv16, 1) * 16)) {
+    lc.grids.clear();
+    if (sizeof(T) == 4) drop_patch_tab(h, h->d.lev[l].X);
+    return IGAMG_OK;
+  }
   int *wdesc, *wspec, rc;
   if ((rc = upload_as(h, &wdesc, G.wdesc)) || (rc = upload_as(h, &wspec, G.wspec))) return rc;
   X.gcls = lc.gcls;
@@ -1731,7 +1757,6 @@ int build_patch_tab(igamg_handle* h, int l, TypedLevel<T>& tl) {
     k_patch_ext<P, T><<<nblk(n), kBlock, 0, h->stream>>>(n, L.n_ux, L.sext, ext);
     X.ext = ext;
   }
-  const int n8 = std::max(lh.pt.n_cls8, 1), nw = (int)G.wspec.size() / 4;
   if ((rc = dmalloc(h, (void**)&inv8, (size_t)n8 * 8 * inv8_ld<T>() * sizeof(E))) ||
       (rc = dmalloc(h, (void**)&winv, (size_t)std::max(G.winv16, 1) * 16)))
     return rc;
@@ -1741,6 +1766,17 @@ int build_patch_tab(igamg_handle* h, int l, TypedLevel<T>& tl) {
   X.inv8 = inv8;
   X.winv = winv;
   return launch_check();
+}
+
+// Frees the local inverses that only the row kernels and the fused coarse end read, on the levels
+// that run neither (known once the sweep forms and the coarse end are chosen).
+template <typename T>
+void drop_row_inverses(igamg_handle* h, Typed<T>& ty) {
+  for (int l = std::max(1, ty.fused_lc + 1); l < (int)ty.lev.size(); ++l)
+    if (h->lc[l].staged) {
+      dfree(h, ty.lev[l].cinv);
+      dfree(h, ty.lev[l].cinv8);
+    }
 }
 
 // Upload the typed (double or float) copy of every level's tables and workspaces.
@@ -2301,6 +2337,9 @@ int igamg_create(const igamg_problem* prob, void* cuda_stream, igamg_handle** ou
   if (!h->host.jt.empty() && (rc = upload_as(h, &h->jt, h->host.jt))) return fail(rc);
   if ((rc = autotune_fused<double>(h, h->d))) return fail(rc);
   if (fp32_base(pr) && (rc = autotune_fused<float>(h, h->f))) return fail(rc);
+  if (cudaStreamSynchronize(h->stream) != cudaSuccess) return fail(IGAMG_ECUDA);
+  drop_row_inverses<double>(h, h->d);
+  if (fp32_base(pr)) drop_row_inverses<float>(h, h->f);
   if (pr.precision >= IGAMG_FGMRES_FP64 &&
       (rc = krylov_alloc(h->kw, pr.restart > 0 ? pr.restart : 20, nfine, h->allocs)))
     return fail(rc);

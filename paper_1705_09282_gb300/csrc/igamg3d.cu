@@ -267,6 +267,15 @@ int dmalloc(igamg3d_handle* h, void** p, size_t bytes) {
   return IGAMG_OK;
 }
 
+// Frees one of the handle's allocations early.
+template <typename V>
+void dfree(igamg3d_handle* h, V*& p) {
+  if (!p) return;
+  h->allocs.erase(std::find(h->allocs.begin(), h->allocs.end(), (void*)p));
+  cudaFree((void*)p);
+  p = nullptr;
+}
+
 template <typename V, typename S>
 int upload_as(igamg3d_handle* h, V** dst, const std::vector<S>& src) {
   std::vector<V> tmp(src.begin(), src.end());
@@ -311,8 +320,16 @@ template <typename T> Typed3<T>& typed(igamg3d_handle* h);
 template <> Typed3<double>& typed<double>(igamg3d_handle* h) { return h->d; }
 template <> Typed3<float>& typed<float>(igamg3d_handle* h) { return h->f; }
 
+template <typename Tab, typename H>
+void drop_patch_tab(H* h, Tab& X) {
+  dfree(h, X.rec);
+  dfree(h, X.ext);
+  dfree(h, X.inv8);
+  dfree(h, X.winv);
+}
+
 // The staged patch kernels' tables of level l, made on the device from the uploaded ones.  Sets
-// lc.staged if the level suits those kernels.
+// lc.staged if the level suits those kernels and memory is not short (staged_fits).
 template <int P, typename T>
 int build_patch_tab3(igamg3d_handle* h, int l, Lev3T<T>& tl) {
   using E = limb_t<T>;
@@ -329,6 +346,14 @@ int build_patch_tab3(igamg3d_handle* h, int l, Lev3T<T>& tl) {
   PatchGrids3 G;
   X.by_row = L.srow != nullptr;
   if (!patch_grids3(P, hl.sz, hl.pt, hl.st, X.koff, X.by_row, (int)sizeof(E), G)) { lc.staged = false; return IGAMG_OK; }
+  const size_t rows = L.srow ? (size_t)L.n_total - 1 : (size_t)total;
+  const size_t next = L.sext ? (size_t)2 * L.n_uc * ext3_rec_len<P, T>() : 0;
+  if (!staged_fits((rows * rec3_len<P, T>() + next + (size_t)std::max(hl.pt.n_cls8, 1) * 8 * inv8_ld<T>()) * sizeof(E) +
+                   (size_t)std::max(G.winv16, 1) * 16)) {
+    lc.staged = false;
+    if (sizeof(T) == 4) drop_patch_tab(h, h->d.lev[l].X);
+    return IGAMG_OK;
+  }
   lc.staged = true;
   lc.grids.clear();
   for (const PatchGrid3& g : G.colour) {
@@ -380,6 +405,18 @@ int build_patch_tab3(igamg3d_handle* h, int l, Lev3T<T>& tl) {
   X.inv8 = inv8;
   X.winv = winv;
   return launch_check();
+}
+
+// Frees the local inverses that only the row kernels and the cluster form read, on the levels that
+// run neither (known once the cluster depth is chosen).
+template <typename T>
+void drop_row_inverses(igamg3d_handle* h, Typed3<T>& ty) {
+  for (int l = std::max(1, ty.fused_lc + 1); l < (int)ty.lev.size(); ++l)
+    if (h->lc[l].staged) {
+      dfree(h, ty.lev[l].cinv);
+      dfree(h, ty.lev[l].cinv8);
+      dfree(h, ty.lev[l].cinv_all);
+    }
 }
 
 // Levels that suit the staged patch kernels use them (measured faster on every level; figures in
@@ -954,6 +991,9 @@ int h3_create(const igamg_problem* prob, void* cuda_stream, igamg3d_handle** out
   // the cluster tuner runs V-cycles: only once every workspace above exists
   if ((rc = setup_cluster3<double>(h, h->d))) return fail(rc);
   if (fp32_base3(pr) && (rc = setup_cluster3<float>(h, h->f))) return fail(rc);
+  if (cudaStreamSynchronize(h->stream) != cudaSuccess) return fail(IGAMG_ECUDA);
+  drop_row_inverses<double>(h, h->d);
+  if (fp32_base3(pr)) drop_row_inverses<float>(h, h->f);
   if (pr.precision >= IGAMG_FGMRES_FP64) {
     if ((rc = krylov_alloc(h->kw, pr.restart > 0 ? pr.restart : 20, nfine, h->allocs))) return fail(rc);
     if ((rc = dmalloc(h, (void**)&h->zeros, nfine * sizeof(double)))) return fail(rc);

@@ -49,6 +49,8 @@
 // 256^2 11.1 -> 7.6; generalized Oseen 512^2 V-cycle 2908 -> 1966 us.  FP32 (same staging, FP32
 // arithmetic): p = 2 4.1 -> 1.5-1.8 us, p = 3 7.6 -> 1.3-1.6.
 #pragma once
+#include <cstdlib>
+
 #include "kernels.cuh"
 
 namespace igamg {
@@ -95,6 +97,18 @@ template <typename T> constexpr int inv8_ld() { return sizeof(T) == 8 ? 10 : 8; 
 // row length of a packed inverse of nl rows: odd, so that the rows of a warp fall into different
 // banks; the FP64 exponents are the entry after the nl-th (3D)
 __host__ __device__ constexpr int wall_ld(int nl) { return (nl + 1) | 1; }
+
+// The staged tables repeat a level's operator records (which the residual goes on reading) and its
+// local inverses: 976 against 944 bytes a row in 3D at p = 2, 5008 against 3808 at p = 3, 640 against 512
+// bytes per interior patch.  A level takes them only if as much device memory stays free as they fill, so that a
+// problem that fits without them still does; it runs the row kernels then.  IGAMG_STAGED_FREE: the
+// bytes taken as free (tests).
+inline bool staged_fits(size_t bytes) {
+  size_t left = 0, total = 0;
+  if (const char* e = std::getenv("IGAMG_STAGED_FREE")) left = (size_t)std::strtoull(e, nullptr, 10);
+  else if (cudaMemGetInfo(&left, &total) != cudaSuccess) { cudaGetLastError(); return true; }
+  return bytes <= left / 2;
+}
 
 // One colour's patches (PatchGrid, igamg_internal.h).
 struct ColourGrid {

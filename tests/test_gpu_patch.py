@@ -244,3 +244,75 @@ def test_3d_records_read_in_place_equal_records_fetched_ahead(p, n, kind, monkey
         assert float((out[0] - out[1]).abs().max()) <= 5e-5 * float(out[1].abs().max())
     else:
         assert torch.equal(out[0], out[1])
+
+
+def _staged(S):
+    import ctypes
+
+    from paper_1705_09282_gb300 import _lib
+    U, R = S.empty(), S.empty()
+    rc = _lib.lib().igamg_probe_patch_rows(S._h, 1, ctypes.c_void_p(U.data_ptr()), ctypes.c_void_p(U.data_ptr()),
+                                           ctypes.c_void_p(R.data_ptr()))
+    return rc == 0
+
+
+@pytest.mark.parametrize("kind,p,n,dim", [("oseen", 2, 16, 2), ("annulus", 3, 16, 2), ("oseen", 2, 8, 3), ("cylinder-fp32", 2, 6, 3)])
+def test_levels_without_memory_for_staged_tables_run_the_row_kernels(kind, p, n, dim, monkeypatch):
+    torch = _torch()
+    from paper_1705_09282_gb300 import _lib
+    from paper_1705_09282_gb300.solver import Solver
+    kw = {"dim": 3} if dim == 3 else {}
+    if kind == "oseen":
+        kw["beta"] = inputs.oseen_advection_3d(p, n, 0.5) if dim == 3 else inputs.oseen_advection(p, n, 0.5)
+    else:
+        kw["geometry"] = _lib.IGAMG_GEOM_QUARTER_ANNULUS if dim == 2 else _lib.IGAMG_GEOM_HOLLOW_CYLINDER
+    if kind.endswith("fp32"):
+        kw["precision"] = _lib.IGAMG_FP32_IR
+    monkeypatch.setenv("IGAMG_FUSED_LEVELS", "-1")
+    out = []
+    for free in (None, "0"):
+        if free is not None:
+            monkeypatch.setenv("IGAMG_STAGED_FREE", free)
+        S = Solver(p, n, 2, 10.0, 0.5, **kw)
+        assert _staged(S) == (free is None)
+        F = torch.tensor(inputs.random_vector(S.ndof(), seed=n + 1), device="cuda")
+        V = S.empty()
+        S.vcycle(V, F)
+        out.append(V.clone())
+        S.close()
+    tol = 5e-5 if kind.endswith("fp32") else 1e-11            # four sweeps and a coarse solve of the sweeps' 1e-12
+    assert float((out[0] - out[1]).abs().max()) <= tol * float(out[0].abs().max())
+
+
+def test_staged_levels_hold_their_local_inverses_once(monkeypatch):
+    # an operator with records and inverses per row and patch: the staged handle holds more than the row
+    # kernels' one by its records (976 bytes a row), the wall patches' rows (64 entries of 16 bytes each) and
+    # the padding of its inverses (8 to 10 entries a row of the 8 x 8 ones, under 12 % on the others), not by a
+    # second copy of the inverses
+    torch = _torch()
+    from paper_1705_09282_gb300.solver import Solver
+    n, L = 24, 3
+    beta = inputs.oseen_advection_3d(2, n, 0.5)
+    monkeypatch.setenv("IGAMG_FUSED_LEVELS", "-1")
+
+    def held(form):
+        if form:
+            monkeypatch.setenv("IGAMG_SWEEP_FORM", form)
+        else:
+            monkeypatch.delenv("IGAMG_SWEEP_FORM", raising=False)
+        torch.cuda.synchronize()
+        before = torch.cuda.mem_get_info()[0]
+        S = Solver(2, n, L, 10.0, 0.5, dim=3, beta=beta)
+        used = before - torch.cuda.mem_get_info()[0]
+        rows = sum(S.ndof(l) for l in range(L))
+        staged = _staged(S)
+        S.close()
+        return used, rows, staged
+
+    held(None)                                                # loads the kernels
+    used, rows, staged = held(None)
+    base, _, rowform = held("rows")
+    assert staged and not rowform
+    inverses = base - 944 * rows
+    walls = sum(3 * (m + 1) * m ** 2 - 3 * (m - 3) * (m - 4) ** 2 for m in (n, n // 2))
+    assert used <= base + 976 * rows + 1024 * walls + 0.25 * inverses + (8 << 20)
