@@ -1556,15 +1556,18 @@ int setup_fused(igamg_handle* h, Typed<T>& ty) {
 struct TuneKey {
   int p, n, L, bytes, sm, nu1, nu2;
   int rows;                     // 1: per-row operators (Oseen, mapped domains), 0: class stencils
+  int staged;                   // bit l: level l runs the staged patch solves, against which the depths are timed
   bool operator<(const TuneKey& o) const {
-    return std::tie(p, n, L, bytes, sm, nu1, nu2, rows) < std::tie(o.p, o.n, o.L, o.bytes, o.sm, o.nu1, o.nu2, o.rows);
+    return std::tie(p, n, L, bytes, sm, nu1, nu2, rows, staged) <
+           std::tie(o.p, o.n, o.L, o.bytes, o.sm, o.nu1, o.nu2, o.rows, o.staged);
   }
 };
 std::map<TuneKey, std::pair<int, int>>& tune_cache() { static std::map<TuneKey, std::pair<int, int>> m; return m; }
 std::mutex& tune_mutex() { static std::mutex m; return m; }
 
 // IGAMG_TUNE_CACHE=<file>: the tuned coarse-end choices persist across processes, one line per
-// shape ("p n_fine levels bytes smoother nu1 nu2 rows depth kind"), so that a run under a
+// shape ("v2 p n_fine levels bytes smoother nu1 nu2 rows staged depth kind"; lines of another form,
+// as those tuned against the row kernels alone, are passed over), so that a run under a
 // profiler reuses what a plain run measured (the profiler's serialised launches would skew a
 // fresh tuning).  The file is advisory: unreadable or missing means tune as usual.  Call with
 // tune_mutex held.
@@ -1578,9 +1581,11 @@ void tune_file_load() {
   if (!f) return;
   TuneKey k{};
   int d = 0, kind = 0;
-  while (std::fscanf(f, "%d %d %d %d %d %d %d %d %d %d", &k.p, &k.n, &k.L, &k.bytes, &k.sm, &k.nu1, &k.nu2, &k.rows, &d,
-                     &kind) == 10)
-    tune_cache()[k] = {d, kind};
+  char line[256];
+  while (std::fgets(line, sizeof(line), f))
+    if (std::sscanf(line, "v2 %d %d %d %d %d %d %d %d %d %d %d", &k.p, &k.n, &k.L, &k.bytes, &k.sm, &k.nu1, &k.nu2, &k.rows,
+                    &k.staged, &d, &kind) == 11)
+      tune_cache()[k] = {d, kind};
   std::fclose(f);
 }
 
@@ -1589,7 +1594,8 @@ void tune_file_append(const TuneKey& k, int d, int kind) {
   if (!path) return;
   FILE* f = std::fopen(path, "a");
   if (!f) return;
-  std::fprintf(f, "%d %d %d %d %d %d %d %d %d %d\n", k.p, k.n, k.L, k.bytes, k.sm, k.nu1, k.nu2, k.rows, d, kind);
+  std::fprintf(f, "v2 %d %d %d %d %d %d %d %d %d %d %d\n", k.p, k.n, k.L, k.bytes, k.sm, k.nu1, k.nu2, k.rows, k.staged, d,
+               kind);
   std::fclose(f);
 }
 
@@ -1600,7 +1606,8 @@ int autotune_fused(igamg_handle* h, Typed<T>& ty) {
   if (h->prob.gamma > 1) { ty.fused_lc = -1; return IGAMG_OK; }   // W-cycles run level by level
   const int L = h->prob.n_levels;
   TuneKey key{h->prob.p, h->prob.n_fine, L, (int)sizeof(T), h->prob.smoother, h->prob.nu1, h->prob.nu2,
-              (h->prob.beta_qp || h->prob.geometry != IGAMG_GEOM_SQUARE) ? 1 : 0};
+              (h->prob.beta_qp || h->prob.geometry != IGAMG_GEOM_SQUARE) ? 1 : 0, 0};
+  for (int l = 1; l < L && l < 31; ++l) key.staged |= h->lc[l].staged ? 1 << l : 0;
   // fixed choices (tests, experiments): IGAMG_FUSED_LEVELS = depth, IGAMG_FUSED_CLUSTER = blocks
   const char* env = std::getenv("IGAMG_FUSED_LEVELS");
   if (env) {
@@ -1616,7 +1623,11 @@ int autotune_fused(igamg_handle* h, Typed<T>& ty) {
     std::lock_guard<std::mutex> lk(tune_mutex());
     tune_file_load();
     auto it = tune_cache().find(key);
-    if (it != tune_cache().end()) { ty.fused_lc = it->second.first; ty.fused_kind = it->second.second; return IGAMG_OK; }
+    if (it != tune_cache().end() && it->second.first <= (it->second.second > 1 ? ty.cluster_max : ty.fused_max)) {
+      ty.fused_lc = it->second.first;
+      ty.fused_kind = it->second.second;
+      return IGAMG_OK;
+    }
   }
   T* U = ty.lev[L - 1].U;
   T* F = ty.lev[L - 1].F;

@@ -143,3 +143,25 @@ def test_mixed_precision_fmg_3d():
     rep = S.solve(U, F, rtol=1e-8, max_cycles=40)
     assert rep["converged"]
     assert rep["div_inf"] <= 1e-10 * float(U.abs().max())
+
+
+def test_tuned_depths_of_other_sweep_kernels_are_not_reused(tmp_path):
+    # a cache line without the staged levels (tuned against the row kernels) is passed over; the line
+    # that the tuner writes itself is used by the next process
+    _torch()
+    import os
+    import subprocess
+    import sys
+    cache = tmp_path / "tune"
+    cache.write_text("2 32 4 8 0 2 2 0 3 1\n2 32 4 8 1 2 2 0 3 1\n")
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    env = {k: v for k, v in os.environ.items() if not k.startswith("IGAMG_")}
+    env.update(IGAMG_TUNE_CACHE=str(cache), IGAMG_VERBOSE="1", PYTHONPATH=root)
+    code = "from paper_1705_09282_gb300.solver import Solver; Solver(2, 32, 4, 1.0, 1.0).close()"
+    tuned = []
+    for _ in range(2):
+        r = subprocess.run([sys.executable, "-c", code], env=env, capture_output=True, text=True, timeout=300)
+        assert r.returncode == 0, r.stderr
+        tuned.append("chose fused coarse levels" in r.stderr)
+    assert tuned == [True, False]
+    assert [x for x in cache.read_text().splitlines() if x.startswith("v2 2 32 4 8 ")]
