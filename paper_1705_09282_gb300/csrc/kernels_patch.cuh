@@ -45,8 +45,8 @@
 // the launch's own indices, fetched first and before the wait for the previous kernel
 // (programmatic dependent launch), so a colour's chain is: wait, one fetch of U and F, arithmetic.
 // Measured per colour launch (graph replay; row kernels k_mult_colour -> these), FP64: p = 2
-// 8^2-64^2 5.0-5.4 -> 1.9-2.1 us, 128^2 5.4 -> 2.5, 256^2 8.1 -> 5.0; p = 3 10-10.5 -> 2.5-2.7,
-// 256^2 11.1 -> 7.6; generalized Oseen 512^2 V-cycle 2908 -> 1966 us.  FP32 (same staging, FP32
+// 8^2-64^2 5.0-5.4 -> 1.9-2.1 us, 128^2 5.4 -> 2.4, 256^2 8.1 -> 5.0; p = 3 10-10.5 -> 2.5-2.7,
+// 256^2 11.1 -> 7.4; generalized Oseen 512^2 V-cycle 2908 -> 1977 us.  FP32 (same staging, FP32
 // arithmetic): p = 2 4.1 -> 1.5-1.8 us, p = 3 7.6 -> 1.3-1.6.
 #pragma once
 #include <cstdlib>

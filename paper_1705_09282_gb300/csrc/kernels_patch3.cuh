@@ -17,7 +17,8 @@
 // compile-time strides.  Origins: P_a - p along a != f, P_f - (p-1) along f.
 //
 // Measured per colour launch, FP64 Stokes (k_mult_rows3 / k_mult_rows3x -> these): p = 2 8^3 10.0 ->
-// 3.7 us, 16^3 9.8 -> 4.3, 32^3 10.7 -> 10.1, 64^3 42.1 -> 40.3; p = 3 8^3 41.1 -> 18.2, 16^3 47.0 -> 29.3.
+// 3.8 us, 16^3 9.8 -> 4.4, 32^3 10.7 -> 10.3, 64^3 42.1 -> 40.3; p = 3 8^3 41.1 -> 18.6, 16^3 47.0 -> 29.6.
+// (An exponent per component and the rounding of the rows' sums cost 0.1 to 0.4 us of these up to 16^3.)
 // 64^3 is now bound by the staging itself (232 values fetched and converted for the 8 rows of
 // a patch, about 900 instructions a warp), the small levels by one block's chain of latencies.
 #pragma once

@@ -5,9 +5,11 @@
 // divergence-free velocity, the second with a pressure.
 //
 // Weights are held in BF16 for every product (FP32 master copy for the optimizer);
-// activations and accumulation are FP32.  Forward, backward (data and weights), the masked
-// mean-squared loss and Adam are hand-written kernels; tiles of 16 x 16 pixels per block
-// with the input tile (plus halo) and the layer's weights staged in shared memory.
+// accumulation is FP32.  Forward, backward (data and weights), the masked mean-squared loss and
+// Adam are hand-written kernels.  Training keeps FP32 activations: tiles of 16 x 16 pixels per
+// block with the input tile (plus halo) and the layer's weights staged in shared memory.  Inference
+// hands BF16 activations from layer to layer and runs the 32 -> 32 layers on the tensor cores,
+// over tiles of 128 consecutive pixels whose neighbourhoods are gathered from global memory.
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
